@@ -51,19 +51,31 @@ cudaError_t dev_alloc(void** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 
-int grid_blocks(int64_t n, int threads, int waves) {
-  static int sm_count[64] = {0};
+static int sm_count() {
+  static int counts[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
-  int& sms = sm_count[dev & 63];
+  int& sms = counts[dev & 63];
   if (sms == 0) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
       sms = 1;
   }
+  return sms;
+}
+
+static int capped_blocks(int64_t n, int threads, int64_t cap) {
   const int64_t need = (n + threads - 1) / threads;
-  const int64_t cap = (int64_t)sms * (2048 / threads) * waves;   // some waves, then grid-stride
   const int64_t b = need < cap ? need : cap;
   return (int)(b < 1 ? 1 : b);
+}
+
+int grid_blocks(int64_t n, int threads, int waves) {
+  // some waves, then grid-stride
+  return capped_blocks(n, threads, (int64_t)sm_count() * (2048 / threads) * waves);
+}
+
+int queue_blocks(int64_t n, int threads, int per_sm) {
+  return capped_blocks(n, threads, (int64_t)sm_count() * per_sm);
 }
 
 bool handle_ok(stf_texture t) {

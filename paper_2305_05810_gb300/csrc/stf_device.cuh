@@ -282,6 +282,27 @@ __device__ __forceinline__ bool misses(const MissBox& m, const float* x) {
          x[2] >= m.hi[2];
 }
 
+// The coordinates whose window floor(x) + LO .. floor(x) + HI reaches into [lo, hi) on
+// every axis (the complement of MissBox, for any window).  NaN and infinities are outside;
+// a bound beyond +-2^24 is open, because finite coordinates beyond 2^24 are clamped to it.
+struct LiveBox {
+  float lo[3], hi[3];
+  __device__ __forceinline__ bool has(const float* x) const {
+    return x[0] >= lo[0] && x[0] < hi[0] && x[1] >= lo[1] && x[1] < hi[1] && x[2] >= lo[2] && x[2] < hi[2];
+  }
+};
+
+__device__ __forceinline__ LiveBox live_box(const int* lo, const int* hi, int LO, int HI) {
+  LiveBox b;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int l = lo[a] - HI, h = hi[a] - LO;
+    b.lo[a] = l <= -16777216 ? -3.402823466e38f : __int2float_ru(l);
+    b.hi[a] = h > 16777216 ? __int_as_float(0x7f800000) : __int2float_ru(h);
+  }
+  return b;
+}
+
 // ---------------------------------------------------------------- views
 struct Tex2DView {
   const void* texels;     // storage format, [level][y][x][c]; DCT6: [level][by][bx][c] words
@@ -381,6 +402,52 @@ __device__ __forceinline__ void quad_loop3_joint(const LookupArgs& a, Quad quad,
   }
   for (uint32_t i = 4 * groups + tid; i < n; i += stride)
     a.out[i] = one(__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2), i);
+}
+
+// A warp's chunks of SIZE queries: one of every row of (warps x SIZE) queries, at a place
+// that moves on by the golden section of the row each time.  With a fixed place, warps
+// whose stride is near a multiple of an image's rows met one column of it only, and those
+// on the columns that cross the grid ran on alone (half of the sparse filter's time).
+template <int SIZE>
+struct WarpChunks {
+  uint32_t row, place, warps, turn;
+  __device__ __forceinline__ WarpChunks() {
+    warps = gridDim.x * (blockDim.x / 32);
+    place = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    turn = (uint32_t)(0.6180339887f * (float)warps);
+    row = 0;
+  }
+  __device__ __forceinline__ uint32_t first() const { return row + place * SIZE; }
+  __device__ __forceinline__ void next() {
+    row += warps * SIZE;
+    place += turn;
+    if (place >= warps) place -= warps;
+  }
+};
+
+// Coordinates of the queries i0 .. i0 + PER - 1 (NaN past the end), whose results are set
+// to the background: three 16-byte loads and one store for four queries of aligned arrays.
+template <int PER>
+__device__ __forceinline__ void load_and_clear(const LookupArgs& a, float background, bool aligned, uint32_t i0,
+                                               uint32_t n, float (&x)[PER][3]) {
+  if (PER == 4 && aligned && i0 + PER <= n) {
+    const float4* c4 = reinterpret_cast<const float4*>(a.coords) + 3 * (i0 / 4);
+    const float4 p = __ldg(c4), q = __ldg(c4 + 1), r = __ldg(c4 + 2);
+    const float v[12] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w, r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int k = 0; k < 3 * PER; ++k) x[k / 3][k % 3] = v[k];
+    reinterpret_cast<float4*>(a.out)[i0 / 4] = make_float4(background, background, background, background);
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    x[k][0] = x[k][1] = x[k][2] = __int_as_float(0x7fc00000);
+    if (i0 + k < n) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[k][d] = __ldg(a.coords + 3 * (i0 + k) + d);
+      a.out[i0 + k] = background;
+    }
+  }
 }
 
 __device__ __forceinline__ int64_t query_slot(const LookupArgs& a, int64_t i) {

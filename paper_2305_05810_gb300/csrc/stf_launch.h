@@ -11,12 +11,27 @@ enum Op { OP_STOCHASTIC = 0, OP_DETERMINISTIC = 1, OP_ACCUMULATE = 2 };
 // Grid size for a grid-stride launch: enough blocks for n, capped at `waves` full waves
 // of 2048 threads per SM.
 int grid_blocks(int64_t n, int threads, int waves = 4);
+// Grid size for kernels whose warps keep queues: at most the blocks that are resident at
+// once (`per_sm` on each SM), so that few warps end with partly filled queues.
+int queue_blocks(int64_t n, int threads, int per_sm);
 // The stochastic dense and sparse kernels launch up to 8 waves of 256-thread blocks.
 // With four queries per thread and the miss shortcut, 8 waves finished the dense
 // benchmark call 3% sooner than 16 and 6% sooner than 32 (2: 11% later; 4 and 6 within
 // 1% of 8, sparse 1-5% slower).  The 2D kernels keep 4 waves (no gain at 16.8M queries,
 // 3% slower at 5.3M with 16).
 constexpr int kStochasticWaves = 8;
+
+// Deterministic 3D calls of at least this many queries take chunks of 128 per warp (three
+// 16-byte coordinate loads per lane, fuller queues); below it chunks of 32 spread a
+// call over more warps.
+constexpr int64_t kQueueChunkMin = 1 << 20;
+
+// The filter whose deterministic form filter F has.
+constexpr int deterministic_filter(int F) {
+  return F == STF_FILTER_FIS_LINEAR ? STF_FILTER_LINEAR
+         : F == STF_FILTER_FIS_BSPLINE3 ? STF_FILTER_BSPLINE3
+         : F == STF_FILTER_CATMULL_ROM_POSITIVIZED ? STF_FILTER_CATMULL_ROM : F;
+}
 
 cudaError_t launch_tex2d(Op op, int filter, int fmt, int channels, const Tex2DView& t,
                          const LookupArgs& a, cudaStream_t s);
