@@ -770,13 +770,10 @@ __device__ __forceinline__ float dct_ac(uint32_t w, int j) {
   return (float)(((int32_t)(w << (20 - 5 * j))) >> 27);     // 5-bit field, sign-extended
 }
 
-// Texel (x, y) of level L, clamped to the level: f = sum over the six coefficients of
-// value * basis(x) * basis(y), float32.
+// The code words (one per channel) of the block that starts at `word` of the texture.
 template <int C>
-__device__ __forceinline__ void dct_texel(const Tex2DView& t, int L, int x, int y, float* v) {
-  const uint32_t* p = reinterpret_cast<const uint32_t*>(t.texels) + t.level_off[L] +
-                      ((int64_t)(y >> 3) * t.blocks_w[L] + (x >> 3)) * C;
-  uint32_t w[C];
+__device__ __forceinline__ void dct_codes(const Tex2DView& t, int64_t word, uint32_t* w) {
+  const uint32_t* p = reinterpret_cast<const uint32_t*>(t.texels) + word;
   if constexpr (C % 4 == 0) {
 #pragma unroll
     for (int k = 0; k < C / 4; ++k) {
@@ -789,12 +786,13 @@ __device__ __forceinline__ void dct_texel(const Tex2DView& t, int L, int x, int 
   } else {
     w[0] = __ldg(p);
   }
-  float x0, x1, x2, y0, y1, y2;
-  dct_basis(t, x & 7, x0, x1, x2);
-  dct_basis(t, y & 7, y0, y1, y2);
-  // DC code step folded into its basis product; each channel's AC step multiplies the
-  // sum of its five integer codes times their basis products
-  const float b[6] = {x0 * y0 * (8.0f / 127.0f), x1 * y0, x0 * y1, x2 * y0, x1 * y1, x0 * y2};
+}
+
+// Values of a block's codes for the basis products b: f = sum over the six coefficients
+// of value * b, float32.  The DC code step is folded into b[0]; each channel's AC step
+// multiplies the sum of its five integer codes times their basis products.
+template <int C>
+__device__ __forceinline__ void dct_decode(const Tex2DView& t, const uint32_t* w, const float* b, float* v) {
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     float ac = dct_ac(w[c], 0) * b[1];
@@ -802,6 +800,18 @@ __device__ __forceinline__ void dct_texel(const Tex2DView& t, int L, int x, int 
     for (int j = 1; j < 5; ++j) ac = fmaf(dct_ac(w[c], j), b[j + 1], ac);
     v[c] = fmaf(t.ac_step[c], ac, (float)(w[c] & 127u) * b[0]);
   }
+}
+
+// Texel (x, y) of level L, clamped to the level.
+template <int C>
+__device__ __forceinline__ void dct_texel(const Tex2DView& t, int L, int x, int y, float* v) {
+  uint32_t w[C];
+  dct_codes<C>(t, t.level_off[L] + ((int64_t)(y >> 3) * t.blocks_w[L] + (x >> 3)) * C, w);
+  float x0, x1, x2, y0, y1, y2;
+  dct_basis(t, x & 7, x0, x1, x2);
+  dct_basis(t, y & 7, y0, y1, y2);
+  const float b[6] = {x0 * y0 * (8.0f / 127.0f), x1 * y0, x0 * y1, x2 * y0, x1 * y1, x0 * y2};
+  dct_decode<C>(t, w, b, v);
 }
 
 // Texel (cx, cy) of level L, already clamped to the level, in any 2D storage format.

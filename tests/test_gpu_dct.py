@@ -259,3 +259,22 @@ def test_full_size_dct_plane_sampled():
     err = np.abs(gv - rv)[ok]
     assert np.all(err <= _decode_tol(ref) + 2e-6 * np.abs(rv[ok])), np.max(err)
     stf.stf_synchronize(T.handle)
+
+
+@pytest.mark.parametrize("channels", [1, 2, 4, 8])
+@pytest.mark.parametrize("filt", ["linear", "bspline3", "catmull_rom"])
+def test_deterministic_windows_across_blocks(filt, channels):
+    """Windows inside one 8x8 block and across two or four, clamped at the edges, at sizes
+    that are no multiple of 8 and at warps that are not full: the block-wise decode against
+    the oracle's texel-wise sum."""
+    T, ref, _ = _dct_pair(W=38, H=22, C=channels, levels=2, seed=20 + channels)
+    u = (np.arange(38 * 4 + 9, dtype=np.float32) - 4) / np.float32(38 * 4)
+    v = (np.arange(22 * 2 + 5, dtype=np.float32) - 2) / np.float32(22 * 2)
+    uv = np.stack(np.meshgrid(u, v, indexing="ij"), -1).reshape(-1, 2).astype(np.float32)
+    lod = (synth.uniform(len(uv), 3) * np.float32(1.4)).astype(np.float32)
+    uv[7], lod[40], uv[41, 1] = np.nan, np.inf, 3e7
+    for l in (None, lod):
+        det = T.lookup_deterministic(to_dev(uv), None if l is None else to_dev(l), filter=filt).cpu().numpy()
+        dv, _, _ = filters.lookup_2d(ref, uv, l, filt, stochastic_form=False)
+        # Catmull-Rom weights sum to at most 1.25 per axis in magnitude
+        assert np.all(np.abs(det - dv) <= 1.25 ** 2 * _decode_tol(ref) + 2e-6 * np.abs(dv))
