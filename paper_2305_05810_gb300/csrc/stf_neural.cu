@@ -691,15 +691,6 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
 
 // ---------------------------------------------------------------- training
 
-struct ActBuffers {   // binary16 activations of one batch, row-major
-  __half* x;    // [B][8]
-  __half* h1;   // [B][64]
-  __half* h2;   // [B][64]
-  __half* dy;   // [B][8]
-  __half* da2;  // [B][64]
-  __half* da1;  // [B][64]
-};
-
 struct TrainArgs {
   const int64_t* ids;          // explicit texel ids (gradient check) or NULL
   const float* target_rows;    // explicit targets [B][7] or NULL
@@ -709,6 +700,7 @@ struct TrainArgs {
   uint64_t seed;
   int64_t step;                // training step (permutation position and Adam t)
   float lr, beta1, beta2, eps;
+  float* grads;                // parameter gradients, accumulated (16-byte aligned)
   float* loss;                 // accumulated sum of squared errors / batch
   float* dx_out;               // [B][8] latent gradients (gradient check) or NULL
   int train;                   // 1: Adam update of the latents in place
@@ -748,18 +740,45 @@ __device__ __forceinline__ int64_t permute_index(int64_t x, int64_t n, uint64_t 
 
 // ---------------------------------------------------------------- tcgen05 training
 //
-// Forward and backward of the decoder for tiles of 128 training texels on the
-// fifth-generation tensor cores: six tcgen05.mma round trips per tile (M = 128,
-// binary16 operands in shared memory, float32 accumulators in tensor memory), issued
-// by one thread, each followed by an epilogue in which every thread reads its row:
-//   H1 = ReLU(X W1 + b1), H2 = ReLU(H1 W2 + b2), Y = H2 W3 + b3       (forward)
-//   dY = 2 (Y - T) / B, dA2 = (dY W3^T) [H2 > 0], dA1 = (dA2 W2^T) [H1 > 0],
-//   dX = dA1 W1^T                                                      (backward)
-// The biases enter the forward MMAs as an extra K chunk against columns of ones, as in
-// the decode.  The activations of the batch go to global memory for the weight
-// gradients; the latents take an Adam step (training) or their gradients are returned.
+// Forward and backward of the decoder and the parameter gradients for tiles of 128
+// training texels on the fifth-generation tensor cores: six tcgen05.mma round trips per
+// tile (M = 128, binary16 operands in shared memory, float32 accumulators in tensor
+// memory), issued by one thread of a 128-thread group, each followed by an epilogue in
+// which every thread reads its row:
+//   1  H1 = ReLU(X W1 + b1)
+//   2  H2 = ReLU(H1 W2 + b2)
+//   3  Y = H2 W3 + b3, dY = 2 (Y - T) / B
+//   4  dA2 = (dY W3^T) [H2 > 0]        and  [H1 | H2]^T dY    : dW3 in rows 64..127
+//   5  dA1 = (dA2 W2^T) [H1 > 0]       and  [H1 | dA2]^T dA2  : dW2 in rows 0..63
+//   6  dX = dA1 W1^T                   and  [dA1 | dA2]^T [X | 1] : dW1^T in rows 0..63,
+//                                           db1 and db2 in the column of ones
+// The gradients' reduction runs over the batch, the rows of the tiles: the tiles that are
+// K-major operands of the layers are read as MN-major ones there, so nothing is
+// transposed or written to memory.  dA2 and dA1 replace H2 and H1 in place once step 4
+// and step 5 have read them.  The gradient accumulators stay in tensor memory over a
+// group's tiles; the groups' sums meet in shared memory and one vector atomic add per
+// four entries takes a CTA's to memory.  The biases enter the forward MMAs as an extra K
+// chunk against columns of ones, as in the decode.
+//
+// A group takes 160 tensor-memory columns (64 for the layers, 96 for the gradients) and
+// 40 KB of tiles: three groups fill an SM's 512 columns, and their waits overlap.  Per
+// 65,536 texels (1024^2 texture): 33 us for the two passes and 54 us for a separate kernel that
+// read the activations back and transposed them in shared memory, 30 us fused; bound by the
+// latency of the six round trips and of the gathers.
 
 namespace tct {
+
+constexpr int GROUPS = 3;
+constexpr int TMEM_COLS = 512;
+constexpr int COLS = 160, C_W2 = 64, C_W3 = 128, C_W1 = 144;   // a group's columns: D, dW2, dW3, dW1
+
+struct alignas(128) Group {
+  unsigned char x[128 * 16 * 2];       // latents in k 0..7, ones in k 8, 9
+  unsigned char dy[128 * 16 * 2];      // dY in k 0..6, zeros beyond
+  unsigned char h[128 * 128 * 2];      // H1 in k 0..63, H2 in k 64..127; then dA1, dA2
+  uint64_t bar;
+  int abort, tiles;
+};
 
 struct Smem {
   unsigned char b1[tc::B1_BYTES];      // W1^T (64 x 16): k 0..7, biases (hi, lo) in k 8, 9
@@ -771,24 +790,32 @@ struct Smem {
   unsigned char r3[64 * 16 * 2];       // W3 (64 x 16): B of dY W3^T (k = output, < 7)
   unsigned char r2[64 * 64 * 2];       // W2 (64 x 64): B of dA2 W2^T
   unsigned char r1[16 * 64 * 2];       // W1 (16 x 64), rows >= 8 zero: B of dA1 W1^T
-  unsigned char x[128 * 16 * 2];       // latents in k 0..7, ones in k 8, 9
-  unsigned char h1[128 * 64 * 2];
-  unsigned char h2[128 * 64 * 2];
-  unsigned char dy[128 * 16 * 2];      // dY in k 0..6, zeros beyond
-  unsigned char da2[128 * 64 * 2];
-  unsigned char da1[128 * 64 * 2];
-  uint64_t bar;
+  Group grp[GROUPS];
+  float sums[GROUPS * 4][8];           // per warp: db3, loss
   uint32_t tmem;
-  int abort;
 };
+static_assert(offsetof(Smem, grp) % 128 == 0 && offsetof(Group, h) % 128 == 0, "tiles are 128-byte aligned");
 
-constexpr int TMEM_COLS = 64;
+// Descriptor of a tile stored with K columns of 16-bit values per row, read as an
+// MN-major operand (no swizzle) from column c0: M or N runs along the columns (core
+// matrices of 8 columns x 8 rows, 128 bytes apart), K along the rows (8-row groups
+// K/8 * 128 bytes apart).  Rows 16 j .. 16 j + 15 start j * K/8 * 256 bytes further.
+__device__ __forceinline__ uint64_t desc_mn(const unsigned char* tile, int c0, int j, int K) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(tile + (c0 >> 3) * 128 + j * (K / 8) * 256);
+  uint64_t d = (uint64_t)((a & 0x3FFFF) >> 4);
+  d |= (uint64_t)(((K / 8) * 128) >> 4) << 16;     // next 8 rows
+  d |= (uint64_t)(128 >> 4) << 32;                 // next 8 columns
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
+// Both operands MN-major.
+__host__ __device__ constexpr uint32_t idesc_mn(int M, int N) { return tc::idesc(M, N) | (1u << 15) | (1u << 16); }
 
 }  // namespace tct
 
-// Forward hidden epilogue with the row also written to global memory (the batch's
-// activations for the weight gradients): D -> ReLU -> binary16 -> A tile row, grow.
-__device__ __forceinline__ void tc_hidden_keep(uint32_t taddr, unsigned char* tile, int row, uint4* grow) {
+// Forward hidden epilogue: D -> ReLU -> binary16 -> columns c0 .. c0 + 63 of the row.
+__device__ __forceinline__ void tct_hidden(uint32_t taddr, unsigned char* h, int c0, int row) {
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     uint32_t r[32];
@@ -801,70 +828,69 @@ __device__ __forceinline__ void tc_hidden_keep(uint32_t taddr, unsigned char* ti
         const int c = 8 * q + 2 * e;
         asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(w[e]) : "f"(__uint_as_float(r[c + 1])), "f"(__uint_as_float(r[c])));
       }
-      const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(tile + tc::off(row, 32 * half + 8 * q, 64)) = v;
-      if (grow) grow[4 * half + q] = v;
+      *reinterpret_cast<uint4*>(h + tc::off(row, c0 + 32 * half + 8 * q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
 
-// Backward epilogue: D (64 float32) masked by the row of the forward activation tile
-// (kept where the activation is > 0, the ReLU derivative) -> binary16 -> A tile row,
-// and to global memory.
-__device__ __forceinline__ void tc_masked_keep(uint32_t taddr, const unsigned char* mask, unsigned char* tile,
-                                               int row, uint4* grow) {
+// Backward epilogue, in place: D (64 float32), kept where the activation in the row's
+// columns c0 .. c0 + 63 is > 0 (the ReLU derivative), replaces it as binary16.
+__device__ __forceinline__ void tct_masked(uint32_t taddr, unsigned char* h, int c0, int row) {
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     uint32_t r[32];
     tc::tmem_ld<32>(taddr + 32 * half, r);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const uint4 m = *reinterpret_cast<const uint4*>(mask + tc::off(row, 32 * half + 8 * q, 64));
+      uint4* p = reinterpret_cast<uint4*>(h + tc::off(row, c0 + 32 * half + 8 * q, 128));
+      const uint4 m = *p;
       const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
       uint32_t w[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int c = 8 * q + 2 * e;
-        const float2 h = unpack_h2(mw[e]);
-        w[e] = pack_h2(h.x > 0.f ? __uint_as_float(r[c]) : 0.f, h.y > 0.f ? __uint_as_float(r[c + 1]) : 0.f);
+        const float2 a = unpack_h2(mw[e]);
+        w[e] = pack_h2(a.x > 0.f ? __uint_as_float(r[c]) : 0.f, a.y > 0.f ? __uint_as_float(r[c + 1]) : 0.f);
       }
-      const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(tile + tc::off(row, 32 * half + 8 * q, 64)) = v;
-      if (grow) grow[4 * half + q] = v;
+      *p = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
 
-__global__ void __launch_bounds__(128, 2) k_neural_fwd_bwd_tc(NeuralDev nd, TrainArgs ta, ActBuffers act) {
+__global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(NeuralDev nd, TrainArgs ta) {
   extern __shared__ __align__(1024) unsigned char dyn[];
   tct::Smem& s = *reinterpret_cast<tct::Smem*>(dyn);
+  constexpr int NT = 128 * tct::GROUPS;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = tid >> 7, row = tid & 127;
+  tct::Group& G = s.grp[g];
   {
     const uint4* img = reinterpret_cast<const uint4*>(nd.wimg);
     const uint4 z = make_uint4(0, 0, 0, 0);
-    tc::stage_fwd_weights(nd, s.b1, s.b2, s.b3, s.b2x, s.b3x, s.ones, tid, 128);
-    for (int n = tid; n < 64; n += 128) {      // W3 rows (k = output) for dY W3^T
+    tc::stage_fwd_weights(nd, s.b1, s.b2, s.b3, s.b2x, s.b3x, s.ones, tid, NT);
+    for (int n = tid; n < 64; n += NT) {       // W3 rows (k = output) for dY W3^T
       *reinterpret_cast<uint4*>(s.r3 + tc::off(n, 0, 16)) = __ldg(img + (nn::I_W3R + n * 8) / 8);
       *reinterpret_cast<uint4*>(s.r3 + tc::off(n, 8, 16)) = z;
     }
-    for (int e = tid; e < 64 * 8; e += 128) {  // W2 rows for dA2 W2^T
+    for (int e = tid; e < 64 * 8; e += NT) {   // W2 rows for dA2 W2^T
       const int n = e >> 3, kc = e & 7;
       *reinterpret_cast<uint4*>(s.r2 + tc::off(n, 8 * kc, 64)) = __ldg(img + (nn::I_W2R + n * 72 + 8 * kc) / 8);
     }
-    for (int e = tid; e < 16 * 8; e += 128) {  // W1 rows (rows >= 8 zero) for dA1 W1^T
+    for (int e = tid; e < 16 * 8; e += NT) {   // W1 rows (rows >= 8 zero) for dA1 W1^T
       const int n = e >> 3, kc = e & 7;
       *reinterpret_cast<uint4*>(s.r1 + tc::off(n, 8 * kc, 64)) =
           n < 8 ? __ldg(img + (nn::I_W1R + n * 72 + 8 * kc) / 8) : z;
     }
-    *reinterpret_cast<uint4*>(s.x + tc::off(tid, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
-    *reinterpret_cast<uint4*>(s.dy + tc::off(tid, 8, 16)) = z;
+    *reinterpret_cast<uint4*>(G.x + tc::off(row, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
+    *reinterpret_cast<uint4*>(G.dy + tc::off(row, 8, 16)) = z;
   }
-  if (tid == 0) {
-    s.abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.bar)));
+  if (row == 0) {
+    G.abort = G.tiles = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&G.bar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (warp == 0) {
+    // (the tiles' shared memory keeps a second CTA of this kernel off the SM)
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(&s.tmem)), "n"(tct::TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -872,30 +898,33 @@ __global__ void __launch_bounds__(128, 2) k_neural_fwd_bwd_tc(NeuralDev nd, Trai
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = s.tmem;
-  const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);   // this warp's lanes
+  const uint32_t tmem = s.tmem + tct::COLS * g;
+  const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);   // this warp's lanes
   uint32_t parity = 0;
   // make the tiles written so far visible to the tensor cores, let one thread issue
-  // the MMAs, wait for them (bounded), and release every thread to read the result
+  // the MMAs, wait for them (bounded), and release the group to read the result
   auto run = [&](auto issue) -> bool {
     asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (tid == 0) {
+    group_sync(g);
+    if (row == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;");
       issue();
-      tc::commit(&s.bar);
-      if (!tc::wait_bar(&s.bar, parity)) s.abort = 1;
+      tc::commit(&G.bar);
+      if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
     }
     parity ^= 1;
-    __syncthreads();
+    group_sync(g);
     asm volatile("tcgen05.fence::after_thread_sync;");
-    return s.abort == 0;
+    return G.abort == 0;
   };
-  float loss_part = 0.0f;
+  float sums[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // db3, sum of squared errors
   const int64_t ntiles = (ta.batch + 127) / 128;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t r = tile * 128 + tid;
+  const int64_t step = (int64_t)gridDim.x * tct::GROUPS;
+  int64_t tile = blockIdx.x + (int64_t)gridDim.x * g;
+  uint32_t more = 0;                          // 0 for the group's first tile: accumulators start from zero
+  for (; tile < ntiles; tile += step) {
+    const int64_t r = tile * 128 + row;
     const bool live = r < ta.batch;
     int64_t id = 0, epoch = 0;
     float T[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -916,23 +945,20 @@ __global__ void __launch_bounds__(128, 2) k_neural_fwd_bwd_tc(NeuralDev nd, Trai
 #pragma unroll
       for (int k = 0; k < 7; ++k) T[k] = tp[k];
     }
-    const uint4 xh = make_uint4(pack_h2(X[0], X[1]), pack_h2(X[2], X[3]), pack_h2(X[4], X[5]),
-                                pack_h2(X[6], X[7]));
-    *reinterpret_cast<uint4*>(s.x + tc::off(tid, 0, 16)) = xh;
-    if (live) reinterpret_cast<uint4*>(act.x)[r] = xh;
-    // forward
-    if (!run([&] { tc::mma(tmem, tc::desc(s.x, 16), tc::desc(s.b1, 16), tc::idesc(128, 64), 0); })) break;
-    tc_hidden_keep(trow, s.h1, tid, live ? reinterpret_cast<uint4*>(act.h1) + r * 8 : nullptr);
+    *reinterpret_cast<uint4*>(G.x + tc::off(row, 0, 16)) =
+        make_uint4(pack_h2(X[0], X[1]), pack_h2(X[2], X[3]), pack_h2(X[4], X[5]), pack_h2(X[6], X[7]));
+    if (!run([&] { tc::mma(tmem, tc::desc(G.x, 16), tc::desc(s.b1, 16), tc::idesc(128, 64), 0); })) break;
+    tct_hidden(trow, G.h, 0, row);
     if (!run([&] {
           for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.h1 + kk * 256, 64), tc::desc(s.b2 + kk * 256, 64), tc::idesc(128, 64), kk);
+            tc::mma(tmem, tc::desc(G.h + kk * 256, 128), tc::desc(s.b2 + kk * 256, 64), tc::idesc(128, 64), kk);
           tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b2x, 16), tc::idesc(128, 64), 1);
         }))
       break;
-    tc_hidden_keep(trow, s.h2, tid, live ? reinterpret_cast<uint4*>(act.h2) + r * 8 : nullptr);
+    tct_hidden(trow, G.h, 64, row);
     if (!run([&] {
           for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.h2 + kk * 256, 64), tc::desc(s.b3 + kk * 256, 64), tc::idesc(128, 16), kk);
+            tc::mma(tmem, tc::desc(G.h + 1024 + kk * 256, 128), tc::desc(s.b3 + kk * 256, 64), tc::idesc(128, 16), kk);
           tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b3x, 16), tc::idesc(128, 16), 1);
         }))
       break;
@@ -943,29 +969,46 @@ __global__ void __launch_bounds__(128, 2) k_neural_fwd_bwd_tc(NeuralDev nd, Trai
 #pragma unroll
       for (int k = 0; k < 7; ++k) {
         const float e = live ? __uint_as_float(y[k]) - T[k] : 0.0f;
-        loss_part = fmaf(e, e, loss_part);
+        sums[7] = fmaf(e, e, sums[7]);
         d[k] = 2.0f * ta.inv_batch * e;
       }
       d[7] = 0.0f;
-      const uint4 dh = make_uint4(pack_h2(d[0], d[1]), pack_h2(d[2], d[3]), pack_h2(d[4], d[5]),
-                                  pack_h2(d[6], d[7]));
-      *reinterpret_cast<uint4*>(s.dy + tc::off(tid, 0, 16)) = dh;
-      if (live) reinterpret_cast<uint4*>(act.dy)[r] = dh;
+      uint32_t w[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        w[k] = pack_h2(d[2 * k], d[2 * k + 1]);
+        const float2 f = unpack_h2(w[k]);
+        sums[2 * k] += f.x;
+        if (k < 3) sums[2 * k + 1] += f.y;
+      }
+      *reinterpret_cast<uint4*>(G.dy + tc::off(row, 0, 16)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    // backward
-    if (!run([&] { tc::mma(tmem, tc::desc(s.dy, 16), tc::desc(s.r3, 16), tc::idesc(128, 64), 0); })) break;
-    tc_masked_keep(trow, s.h2, s.da2, tid, live ? reinterpret_cast<uint4*>(act.da2) + r * 8 : nullptr);
     if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.da2 + kk * 256, 64), tc::desc(s.r2 + kk * 256, 64), tc::idesc(128, 64), kk);
+          tc::mma(tmem, tc::desc(G.dy, 16), tc::desc(s.r3, 16), tc::idesc(128, 64), 0);
+          for (int j = 0; j < 8; ++j)
+            tc::mma(tmem + tct::C_W3, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.dy, 0, j, 16),
+                    tct::idesc_mn(128, 16), more | j);
         }))
       break;
-    tc_masked_keep(trow, s.h1, s.da1, tid, live ? reinterpret_cast<uint4*>(act.da1) + r * 8 : nullptr);
+    tct_masked(trow, G.h, 64, row);
     if (!run([&] {
           for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.da1 + kk * 256, 64), tc::desc(s.r1 + kk * 256, 64), tc::idesc(128, 16), kk);
+            tc::mma(tmem, tc::desc(G.h + 1024 + kk * 256, 128), tc::desc(s.r2 + kk * 256, 64), tc::idesc(128, 64), kk);
+          for (int j = 0; j < 8; ++j)
+            tc::mma(tmem + tct::C_W2, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.h, 64, j, 128),
+                    tct::idesc_mn(128, 64), more | j);
         }))
       break;
+    tct_masked(trow, G.h, 0, row);
+    if (!run([&] {
+          for (int kk = 0; kk < 4; ++kk)
+            tc::mma(tmem, tc::desc(G.h + kk * 256, 128), tc::desc(s.r1 + kk * 256, 64), tc::idesc(128, 16), kk);
+          for (int j = 0; j < 8; ++j)
+            tc::mma(tmem + tct::C_W1, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.x, 0, j, 16),
+                    tct::idesc_mn(128, 16), more | j);
+        }))
+      break;
+    more = 1;
     float dx[8];
     {
       uint32_t q[8];
@@ -999,185 +1042,90 @@ __global__ void __launch_bounds__(128, 2) k_neural_fwd_bwd_tc(NeuralDev nd, Trai
       }
     }
   }
+  // The groups' gradients: groups 1 and 2 leave their rows in their own tiles, [column]
+  // [row], group 0 adds them to its own and takes them to memory.
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) loss_part += __shfl_xor_sync(0xffffffffu, loss_part, o);
-  if (lane == 0) atomicAdd(ta.loss, loss_part * ta.inv_batch);
+  for (int k = 0; k < 8; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sums[k] += __shfl_xor_sync(0xffffffffu, sums[k], o);
+    if (lane == 0) s.sums[warp][k] = sums[k];
+  }
+  if (row == 0) G.tiles = (int)more;
+  float* stage = reinterpret_cast<float*>(G.h);       // dW2 64 x 64, then dW3 or dW1 and db 9 x 128
+  const bool upper = row >= 64;
+  uint32_t v[32];
+  if (g > 0 && more && G.abort == 0) {
+#pragma unroll
+    for (int cb = 0; cb < 2; ++cb) {
+      tc::tmem_ld<32>(trow + tct::C_W2 + 32 * cb, v);
+      if (!upper)
+#pragma unroll
+        for (int n = 0; n < 32; ++n) stage[(32 * cb + n) * 64 + row] = __uint_as_float(v[n]);
+    }
+    tc::tmem_ld<16>(trow + tct::C_W3, v);
+    tc::tmem_ld<16>(trow + tct::C_W1, v + 16);
+#pragma unroll
+    for (int n = 0; n < 9; ++n) stage[4096 + n * 128 + row] = __uint_as_float(upper && n < 7 ? v[n] : v[16 + n]);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (tid == 0 && s.abort) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  bool aborted = false;
+#pragma unroll
+  for (int k = 0; k < tct::GROUPS; ++k) aborted = aborted || s.grp[k].abort;
+  if (g == 0 && more && !aborted) {                    // (group 0 has a tile if any has)
+    auto others = [&](int at) {
+      float a = 0.0f;
+#pragma unroll
+      for (int k = 1; k < tct::GROUPS; ++k)
+        if (s.grp[k].tiles) a += reinterpret_cast<const float*>(s.grp[k].h)[at];
+      return a;
+    };
+#pragma unroll
+    for (int cb = 0; cb < 2; ++cb) {
+      tc::tmem_ld<32>(trow + tct::C_W2 + 32 * cb, v);
+      if (!upper)
+#pragma unroll
+        for (int n = 0; n < 32; n += 4) {
+          float q[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) q[e] = __uint_as_float(v[n + e]) + others((32 * cb + n + e) * 64 + row);
+          atomicAdd(reinterpret_cast<float4*>(ta.grads + nn::P_W2 + row * 64 + 32 * cb + n),
+                    make_float4(q[0], q[1], q[2], q[3]));
+        }
+    }
+    tc::tmem_ld<16>(trow + tct::C_W3, v);
+    tc::tmem_ld<16>(trow + tct::C_W1, v + 16);
+#pragma unroll
+    for (int n = 0; n < 9; ++n) {
+      const float q = __uint_as_float(upper && n < 7 ? v[n] : v[16 + n]) + others(4096 + n * 128 + row);
+      if (upper) {
+        if (n < 7) atomicAdd(ta.grads + nn::P_W3 + (row - 64) * 7 + n, q);
+        if (n == 8) atomicAdd(ta.grads + nn::P_B2 + row - 64, q);
+      } else {
+        atomicAdd(ta.grads + (n < 8 ? nn::P_W1 + n * 64 : nn::P_B1) + row, q);
+      }
+    }
+  }
+  if (tid < 8) {
+    float a = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 4 * tct::GROUPS; ++w) a += s.sums[w][tid];
+    if (tid < 7) atomicAdd(ta.grads + nn::P_B3 + tid, a);
+    else atomicAdd(ta.loss, a * ta.inv_batch);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (tid == 0 && aborted) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "n"(tct::TMEM_COLS));
 }
 
-// Weight and bias gradients on the tensor cores.  The batch is the reduction (K)
-// dimension, so each chunk of 128 batch rows is staged transposed (feature-major, K
-// = batch row) into K-major operand tiles, and two accumulating tcgen05.mma chains per
-// chunk sum over the CTA's chunks in tensor memory:
-//   D1 (128 x 80)  = [H1^T; H2^T] [dA2^T; dY^T]^T : dW2 = rows 0..63 x cols 0..63,
-//                                                    dW3 = rows 64..127 x cols 64..70
-//   D2 (128 x 144) = [X^T; 1; 0] [dA1^T; dA2^T; dY^T]^T : dW1 = rows 0..7 x cols 0..63,
-//                                                    db1, db2, db3 = row 8
-// (the other blocks of the products are not used).  One CTA-wide atomic add per
-// gradient entry at the end.
-namespace tcw {
-
-struct Smem {
-  unsigned char a1[128 * 128 * 2];   // H1^T (rows 0..63), H2^T (rows 64..127)
-  unsigned char a2[128 * 128 * 2];   // X^T (rows 0..7), ones (row 8), zeros
-  unsigned char b[144 * 128 * 2];    // dA1^T (rows 0..63), dA2^T (64..127), dY^T (128..143)
-  uint64_t bar;
-  uint32_t tmem;
-  int abort;
-};
-
-constexpr int TMEM_COLS = 256;   // D1 in columns 0..79, D2 in 96..239
-
-}  // namespace tcw
-
-// Element (m, k) of a K-major operand tile with K = 128.
-__device__ __forceinline__ __half* t128(unsigned char* tile, int m, int k) {
-  return reinterpret_cast<__half*>(tile + tc::off(m, k, 128));
-}
-
-__device__ __forceinline__ void scatter_row(unsigned char* tile, int m0, int k, uint4 v) {
-  const __half* h = reinterpret_cast<const __half*>(&v);
-#pragma unroll
-  for (int e = 0; e < 8; ++e) *t128(tile, m0 + e, k) = h[e];
-}
-
-__global__ void __launch_bounds__(128, 2) k_neural_wgrad_tc(ActBuffers act, int64_t batch, float* grads,
-                                                            unsigned* status) {
-  extern __shared__ __align__(1024) unsigned char dyn[];
-  tcw::Smem& s = *reinterpret_cast<tcw::Smem*>(dyn);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  {
-    const uint4 z = make_uint4(0, 0, 0, 0);
-    for (int e = tid; e < 128 * 128 * 2 / 16; e += 128) reinterpret_cast<uint4*>(s.a2)[e] = z;
-  }
-  __syncthreads();
-  *t128(s.a2, 8, tid) = __float2half_rn(1.0f);
-  if (tid == 0) {
-    s.abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.bar)));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(&s.tmem)), "n"(tcw::TMEM_COLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t d1 = s.tmem, d2 = s.tmem + 96;
-  uint32_t parity = 0;
-  int chunks_done = 0;
-  const int64_t nchunks = (batch + 127) / 128;
-  for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    // stage this thread's batch row (zeros beyond the batch) as column k = tid
-    const int64_t r = c * 128 + tid;
-    const bool live = r < batch;
-    const uint4 z = make_uint4(0, 0, 0, 0);
-    const uint4* h1 = reinterpret_cast<const uint4*>(act.h1) + r * 8;
-    const uint4* h2 = reinterpret_cast<const uint4*>(act.h2) + r * 8;
-    const uint4* a2 = reinterpret_cast<const uint4*>(act.da2) + r * 8;
-    const uint4* a1 = reinterpret_cast<const uint4*>(act.da1) + r * 8;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      scatter_row(s.a1, 8 * q, tid, live ? h1[q] : z);
-      scatter_row(s.a1, 64 + 8 * q, tid, live ? h2[q] : z);
-      scatter_row(s.b, 8 * q, tid, live ? a1[q] : z);
-      scatter_row(s.b, 64 + 8 * q, tid, live ? a2[q] : z);
-    }
-    scatter_row(s.a2, 0, tid, live ? reinterpret_cast<const uint4*>(act.x)[r] : z);
-    scatter_row(s.b, 128, tid, live ? reinterpret_cast<const uint4*>(act.dy)[r] : z);
-    scatter_row(s.b, 136, tid, z);
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t acc = (chunks_done > 0 || kk > 0) ? 1u : 0u;
-        // B rows 64..143 start at the 8th 8-row group (2048 bytes per group at K = 128)
-        tc::mma(d1, tc::desc(s.a1 + kk * 256, 128), tc::desc(s.b + 8 * 2048 + kk * 256, 128),
-                tc::idesc(128, 80), acc);
-        tc::mma(d2, tc::desc(s.a2 + kk * 256, 128), tc::desc(s.b + kk * 256, 128), tc::idesc(128, 144), acc);
-      }
-      tc::commit(&s.bar);
-      if (!tc::wait_bar(&s.bar, parity)) s.abort = 1;   // the tiles are restaged only after this
-    }
-    parity ^= 1;
-    ++chunks_done;
-    __syncthreads();
-    if (s.abort) break;
-  }
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (chunks_done > 0 && !s.abort) {
-    const uint32_t lane_off = (uint32_t)(32 * warp) << 16;
-    const int m = tid;                      // accumulator row = thread
-    uint32_t v[32];
-    // D1 columns 0..63: dW2 (rows < 64); columns 64..79: dW3 (rows >= 64)
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb) {
-      tc::tmem_ld<32>(d1 + lane_off + 32 * cb, v);
-      if (m < 64)
-        for (int n = 0; n < 32; ++n) atomicAdd(grads + nn::P_W2 + m * 64 + 32 * cb + n, __uint_as_float(v[n]));
-    }
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb) {
-      tc::tmem_ld<8>(d1 + lane_off + 64 + 8 * cb, v);
-      if (m >= 64)
-        for (int o = 0; o < 8 && 8 * cb + o < 7; ++o)
-          atomicAdd(grads + nn::P_W3 + (m - 64) * 7 + 8 * cb + o, __uint_as_float(v[o]));
-    }
-    // D2 columns 0..63: dW1 (rows < 8), db1 (row 8); 64..127: db2 (row 8); 128..134: db3
-#pragma unroll
-    for (int cb = 0; cb < 4; ++cb) {
-      tc::tmem_ld<32>(d2 + lane_off + 32 * cb, v);
-      for (int n = 0; n < 32; ++n) {
-        const int col = 32 * cb + n;
-        if (m < 8 && col < 64) atomicAdd(grads + nn::P_W1 + m * 64 + col, __uint_as_float(v[n]));
-        if (m == 8) atomicAdd(grads + (col < 64 ? nn::P_B1 + col : nn::P_B2 + col - 64), __uint_as_float(v[n]));
-      }
-    }
-    tc::tmem_ld<8>(d2 + lane_off + 128, v);
-    if (m == 8)
-      for (int o = 0; o < 7; ++o) atomicAdd(grads + nn::P_B3 + o, __uint_as_float(v[o]));
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (tid == 0 && s.abort) atomicOr(status, STF_DEV_MMA_TIMEOUT);
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "n"(tcw::TMEM_COLS));
-}
-
-static cudaError_t launch_wgrad_tc(const ActBuffers& act, int64_t batch, float* grads, unsigned* status,
-                                   cudaStream_t s) {
-  const int smem = (int)sizeof(tcw::Smem) + 1024;
+// Forward, backward and parameter gradients of a batch (ta.grads and ta.loss zero before).
+static cudaError_t launch_train_tc(const NeuralDev& nd, const TrainArgs& ta, cudaStream_t s) {
+  const int smem = (int)sizeof(tct::Smem);
   static bool attr = false;
   if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_neural_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t nchunks = (batch + 127) / 128;
-  // a few chunks per CTA, so that the accumulators' atomic flush is amortised
-  const int64_t want = (nchunks + 3) / 4;
-  const int grid = (int)(want < (int64_t)sms ? (want < 1 ? 1 : want) : (int64_t)sms);
-  k_neural_wgrad_tc<<<grid, 128, smem, s>>>(act, batch, grads, status);
-  return cudaGetLastError();
-}
-
-// Launch of the tcgen05 forward and backward over a batch.
-static cudaError_t launch_fwd_bwd_tc(const NeuralDev& nd, const TrainArgs& ta, const ActBuffers& act,
-                                     cudaStream_t s) {
-  const int smem = (int)sizeof(tct::Smem) + 1024;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_neural_fwd_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(k_neural_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1185,8 +1133,8 @@ static cudaError_t launch_fwd_bwd_tc(const NeuralDev& nd, const TrainArgs& ta, c
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t ntiles = (ta.batch + 127) / 128;
-  const int grid = (int)(ntiles < (int64_t)sms * 2 ? ntiles : (int64_t)sms * 2);
-  k_neural_fwd_bwd_tc<<<grid, 128, smem, s>>>(nd, ta, act);
+  const int grid = (int)(ntiles < (int64_t)sms ? ntiles : (int64_t)sms);
+  k_neural_train_tc<<<grid, 128 * tct::GROUPS, smem, s>>>(nd, ta);
   return cudaGetLastError();
 }
 
@@ -1403,21 +1351,6 @@ stf_status build_neural(stf_texture_s* t, const stf_neural_desc* d, cudaStream_t
   return STF_OK;
 }
 
-static cudaError_t alloc_acts(ActBuffers& act, void** block, int64_t batch) {
-  const size_t rows = (size_t)batch;
-  cudaError_t e = dev_alloc(block, 2 * rows * (8 + 64 + 64 + 8 + 64 + 64));
-  if (e != cudaSuccess) return e;
-  __half* p = (__half*)*block;
-  act.x = p;   p += rows * 8;
-  act.h1 = p;  p += rows * 64;
-  act.h2 = p;  p += rows * 64;
-  act.dy = p;  p += rows * 8;
-  act.da2 = p; p += rows * 64;
-  act.da1 = p;
-  return cudaSuccess;
-}
-
-
 static stf_status neural_handle(stf_texture t) {
   if (!handle_ok(t)) return fail(STF_ERR_INVALID_HANDLE, "unknown texture handle");
   if (t->kind != STF_KIND_NEURAL2D) return fail(STF_ERR_UNSUPPORTED, "not a neural texture");
@@ -1435,29 +1368,23 @@ extern "C" stf_status stf_neural_gradients(stf_texture t, const int64_t* ids, in
   if (st != STF_OK) return st;
   if (batch < 1 || !ids || !target_rows) return fail(STF_ERR_INVALID_ARGUMENT, "need batch >= 1, ids and targets");
   cudaStream_t s = (cudaStream_t)stream;
-  ActBuffers act;
-  void* block = nullptr;
-  cudaError_t e = alloc_acts(act, &block, batch);
-  if (e != cudaSuccess) return fail_cuda(e, "activation buffers");
   TrainArgs ta;
   memset(&ta, 0, sizeof(ta));
   ta.ids = ids;
   ta.target_rows = target_rows;
   ta.batch = batch;
   ta.inv_batch = 1.0f / (float)batch;
-  ta.loss = t->n_loss;
+  // straight into the caller's arrays; the vector atomics need 16-byte alignment
+  const bool direct = d_param_grads && (uintptr_t)d_param_grads % 16 == 0;
+  ta.grads = direct ? d_param_grads : t->n_grads;
+  ta.loss = d_loss ? d_loss : t->n_loss;
   ta.dx_out = d_latent_grads;
-  e = cudaMemsetAsync(t->n_grads, 0, sizeof(float) * nn::NPARAM, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(t->n_loss, 0, sizeof(float), s);
-  if (e == cudaSuccess) {
-    e = launch_fwd_bwd_tc(t->neural, ta, act, s);
-    if (e == cudaSuccess) e = launch_wgrad_tc(act, batch, t->n_grads, t->d_status, s);
-  }
-  if (e == cudaSuccess && d_param_grads)
+  cudaError_t e = cudaMemsetAsync(ta.grads, 0, sizeof(float) * nn::NPARAM, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ta.loss, 0, sizeof(float), s);
+  if (e == cudaSuccess) e = launch_train_tc(t->neural, ta, s);
+  if (e == cudaSuccess && d_param_grads && !direct)
     e = cudaMemcpyAsync(d_param_grads, t->n_grads, sizeof(float) * nn::NPARAM, cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess && d_loss) e = cudaMemcpyAsync(d_loss, t->n_loss, sizeof(float), cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(block);
   return e == cudaSuccess ? STF_OK : fail_cuda(e, "neural gradients");
 }
 
@@ -1474,10 +1401,7 @@ extern "C" stf_status stf_neural_train(stf_texture t, const float* d_target, con
   if (steps < 0) return fail(STF_ERR_INVALID_ARGUMENT, "steps < 0");
   if (steps == 0) return STF_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  ActBuffers act;
-  void* block = nullptr;
-  cudaError_t e = alloc_acts(act, &block, cfg->batch);
-  if (e != cudaSuccess) return fail_cuda(e, "activation buffers");
+  cudaError_t e = cudaSuccess;
   for (int k = 0; k < steps && e == cudaSuccess; ++k) {
     TrainArgs ta;
     memset(&ta, 0, sizeof(ta));
@@ -1490,13 +1414,13 @@ extern "C" stf_status stf_neural_train(stf_texture t, const float* d_target, con
     ta.beta1 = cfg->beta1;
     ta.beta2 = cfg->beta2;
     ta.eps = cfg->eps;
+    ta.grads = t->n_grads;
     ta.loss = t->n_loss;
     ta.train = 1;
     e = cudaMemsetAsync(t->n_grads, 0, sizeof(float) * nn::NPARAM, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(t->n_loss, 0, sizeof(float), s);
     if (e != cudaSuccess) break;
-    e = launch_fwd_bwd_tc(t->neural, ta, act, s);
-    if (e == cudaSuccess) e = launch_wgrad_tc(act, cfg->batch, t->n_grads, t->d_status, s);
+    e = launch_train_tc(t->neural, ta, s);
     if (e != cudaSuccess) break;
     k_neural_adam<<<1, 256, 0, s>>>(t->n_params, t->n_m, t->n_v, t->n_grads, (float)(t->n_step + 1),
                                     cfg->lr_params, cfg->beta1, cfg->beta2, cfg->eps,
@@ -1506,7 +1430,6 @@ extern "C" stf_status stf_neural_train(stf_texture t, const float* d_target, con
     t->n_step += 1;
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(block);
   return e == cudaSuccess ? STF_OK : fail_cuda(e, "neural training");
 }
 

@@ -229,3 +229,33 @@ def test_neural_slim_decode_equals_tap_output_decode(filt, level_mode):
     slim = T.lookup(to_dev(uv), to_dev(lod), filter=filt, seed=8, level_mode=level_mode)
     torch.cuda.synchronize()
     torch.testing.assert_close(slim, ref, rtol=0, atol=0, equal_nan=True)
+
+
+@pytest.mark.parametrize("batch", [1, 32, 127, 129, 128 * 152 + 1, 128 * 456 + 33])
+def test_gradients_by_batch_size(batch):
+    """Batches of one row, ragged tiles, and tiles that reach the second and third group of
+    a CTA and a group's second tile; with the gradients' array aligned to 4 bytes only, and
+    with outputs left out."""
+    T, ref, lat, par, pyr = make_neural(size=32, latent_levels=3, levels=3)
+    rng = np.random.default_rng(batch)
+    ids = rng.integers(0, lat.shape[0], batch).astype(np.int64)
+    tgt = rng.standard_normal((batch, 7)).astype(np.float32)
+    P = stored_params(par)
+    Y, cache = mlp.forward(h16(lat[ids]), P)
+    g = mlp.backward(cache, P, Y, tgt)
+    want = mlp.loss(Y, tgt)
+    n = stf.NEURAL_PARAMS
+    buf = torch.full((n + 1,), 7.0, device=dev())
+    lg = torch.empty((batch, 8), device=dev())
+    loss = torch.empty(1, device=dev())
+    i, t = to_dev(ids), to_dev(tgt)
+    for pg in (buf[:n], buf[1:]):
+        stf.stf_neural_gradients(T.handle, i, batch, t, pg, lg, loss)
+        G = mlp.unflatten(pg.cpu().numpy())
+        for k in mlp.NAMES:
+            assert np.linalg.norm(G[k] - g[k]) <= 2e-2 * np.linalg.norm(g[k]) + 1e-12, k
+        assert np.linalg.norm(lg.cpu().numpy() - g["X"]) <= 2e-2 * np.linalg.norm(g["X"])
+        assert abs(loss.item() - want) <= 2e-3 * want
+    stf.stf_neural_gradients(T.handle, i, batch, t, None, None, loss)
+    assert abs(loss.item() - want) <= 2e-3 * want
+    stf.stf_synchronize(T.handle)
