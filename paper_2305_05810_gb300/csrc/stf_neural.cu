@@ -178,6 +178,14 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
       "l"(a), "l"(b), "r"(id), "r"(acc));
 }
 
+// The same with A in tensor memory: lane = row, each 32-bit column two consecutive k.
+__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(id), "r"(acc));
+}
+
 __device__ __forceinline__ void commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
       (uint32_t)__cvta_generic_to_shared(bar)));
@@ -232,6 +240,11 @@ __device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]));
+}
+
 // The forward weights as K-major no-swizzle B tiles (threads tid, tid + nt, ...):
 // W1^T (64 x 16) with its bias split into binary16 (hi, lo) in k 8, 9; W2^T (64 x 64);
 // W3^T (16 x 64, rows >= 7 zero); the b2 and b3 bias chunks (64 x 16, 16 x 16) with
@@ -274,7 +287,7 @@ __device__ __forceinline__ void stage_fwd_weights(const NeuralDev& nd, unsigned 
 
 struct Group {                       // one tile in flight
   unsigned char a1[A1_BYTES];
-  unsigned char a2[A2_BYTES];          // H1, then H2, then the staged output rows
+  unsigned char a2[A2_BYTES];          // H1, then the staged output rows
   uint64_t bar;
   int abort;
 };
@@ -319,6 +332,34 @@ __device__ __forceinline__ void tc_hidden(uint32_t taddr, unsigned char* a2, int
       *reinterpret_cast<uint4*>(a2 + tc::off(row, 16 * half + 8 * q, 64)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
+}
+
+// The same for the last hidden layer, whose row goes back to tensor memory as layer 3's A
+// operand: in place, 16 columns of D become 8 of A at or below them, so a tile still
+// takes 64 columns (A in 0..31, D3 in 32..47).  Through shared memory the rows took 128 of
+// a tile's 558 wavefronts to write and as much again for the MMA to read, in a decode that
+// the shared-memory pipe bounded (68% busy; now 53%): 16.8 M stochastic lookups 425 us,
+// 382 us this way.
+__device__ __forceinline__ void tc_hidden_tmem(uint32_t taddr) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t r[16], w[8];
+    tc::tmem_ld<16>(taddr + 16 * q, r);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(w[e]) : "f"(__uint_as_float(r[2 * e + 1])), "f"(__uint_as_float(r[2 * e])));
+    tc::tmem_st8(taddr + 8 * q, w);
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;");
+}
+
+// Layer 3 from the A operand in columns 0..31: D3 (128 x 16) in columns 32..47, bias included.
+__device__ __forceinline__ void tc_layer3(uint32_t tmem, const unsigned char* b3, const unsigned char* b3x,
+                                          const unsigned char* ones) {
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk)
+    tc::mma_ts(tmem + 32, tmem + 8 * kk, tc::desc(b3 + kk * 256, 64), tc::idesc(128, 16), kk);
+  tc::mma(tmem + 32, tc::desc_rows_repeated(ones), tc::desc(b3x, 16), tc::idesc(128, 16), 1);
 }
 
 // Named barrier of one 128-thread group.
@@ -416,17 +457,13 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     group_sync(g);
     if (G.abort) break;
     asm volatile("tcgen05.fence::after_thread_sync;");
-    tc_hidden(trow, G.a2, row);
-    asm volatile("fence.proxy.async.shared::cta;");
+    tc_hidden_tmem(trow);
     asm volatile("tcgen05.fence::before_thread_sync;");
     group_sync(g);
-    // layer 3: D[0, 16) = H2 (128 x 64) * W3 (64 x 16); D2 has been read
+    // layer 3: H2 (128 x 64) * W3 (64 x 16)
     if (row == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-        tc::mma(tmem, tc::desc(G.a2 + kk * 256, 64), tc::desc(s.b3 + kk * 256, 64), tc::idesc(128, 16), kk);
-      tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b3x, 16), tc::idesc(128, 16), 1);   // + b3
+      tc_layer3(tmem, s.b3, s.b3x, s.ones);
       tc::commit(&G.bar);
       if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
     }
@@ -437,7 +474,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     float v[8];
     {
       uint32_t r[8];
-      tc::tmem_ld<8>(trow, r);
+      tc::tmem_ld<8>(trow + 32, r);
 #pragma unroll
       for (int k = 0; k < 7; ++k) v[k] = __uint_as_float(r[k]);
     }
@@ -495,8 +532,8 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
 // holds 128 / R queries.  Each thread gathers its tap's latent texel into the A tile
 // (zeros for fallback levels and for taps of queries without a texture value), the
 // three layers run as in the stochastic decode, and each row's output times its
-// weight (the tap weights wx wy times the level weight) is staged in shared memory;
-// the query's first row then sums its R rows.  Fallback levels use the stored texel.
+// weight (the tap weights wx wy times the level weight) is summed over the query's R
+// rows.  Fallback levels use the stored texel.
 namespace tcd {
 
 struct Smem {
@@ -507,7 +544,7 @@ struct Smem {
   unsigned char b3x[16 * 16 * 2];
   unsigned char ones[8 * 16 * 2];
   unsigned char a1[tc::A1_BYTES];
-  unsigned char a2[tc::A2_BYTES];      // H1, then H2, then the weighted output rows
+  unsigned char a2[tc::A2_BYTES];      // H1
   uint64_t bar;
   uint32_t tmem;
   int abort;
@@ -618,7 +655,6 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
   const int Q = 128 / R;                       // queries per tile
   const int qi = tid / R, sub = tid % R, p = sub / T2, tap = sub % T2;
   const int tx = tap % Fl::T, ty = tap / Fl::T;
-  float* stage = reinterpret_cast<float*>(s.a2);
   const int64_t ntiles = (a.n + Q - 1) / Q;
   int64_t tile = blockIdx.x;
   DetRow cur;
@@ -644,17 +680,12 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
           tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b2x, 16), tc::idesc(128, 64), 1);
         }))
       break;
-    tc_hidden(trow, s.a2, tid);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.a2 + kk * 256, 64), tc::desc(s.b3 + kk * 256, 64), tc::idesc(128, 16), kk);
-          tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b3x, 16), tc::idesc(128, 16), 1);
-        }))
-      break;
+    tc_hidden_tmem(trow);
+    if (!run([&] { tc_layer3(tmem, s.b3, s.b3x, s.ones); })) break;
     float v[8];
     {
       uint32_t r[8];
-      tc::tmem_ld<8>(trow, r);
+      tc::tmem_ld<8>(trow + 32, r);
 #pragma unroll
       for (int k = 0; k < 7; ++k) v[k] = __uint_as_float(r[k]);
     }
@@ -667,20 +698,38 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
         v[2 * k + 1] = f.y;
       }
     }
-    // A2 (H2) has been consumed by layer 3: it now stages the weighted rows
+    // Sum of the query's R rows, which are R consecutive lanes: each exchange halves the
+    // channels a lane keeps (8, 4, 2, 1), further ones add single channels; a lane then
+    // holds channels c and c + 1 (R = 4), or channel c (R >= 8).  Summed by one
+    // thread from rows staged in shared memory, the stores' bank conflicts alone were 224
+    // of a tile's 832 wavefronts.
+    v[7] = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 7; ++k) stage[tid * 8 + k] = cur.mode ? cur.w * v[k] : 0.0f;
-    __syncthreads();
-    if (sub == 0 && cur.i < a.n) {
-      float acc[7] = {0, 0, 0, 0, 0, 0, 0};
-      for (int rr = 0; rr < R; ++rr)
+    for (int k = 0; k < 7; ++k) v[k] = cur.mode ? cur.w * v[k] : 0.0f;
+    const bool hi0 = tid & 1, hi1 = tid & 2, hi2 = tid & 4;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) acc[k] += stage[(tid + rr) * 8 + k];
+    for (int k = 0; k < 4; ++k) {
+      const float o = __shfl_xor_sync(0xffffffffu, hi0 ? v[k] : v[k + 4], 1);
+      v[k] = (hi0 ? v[k + 4] : v[k]) + o;
+    }
 #pragma unroll
-      for (int k = 0; k < 7; ++k) a.out[cur.i * 7 + k] = acc[k];
+    for (int k = 0; k < 2; ++k) {
+      const float o = __shfl_xor_sync(0xffffffffu, hi1 ? v[k] : v[k + 2], 2);
+      v[k] = (hi1 ? v[k + 2] : v[k]) + o;
+    }
+    int c = (hi0 ? 4 : 0) + (hi1 ? 2 : 0);
+    if (R >= 8) {
+      const float o = __shfl_xor_sync(0xffffffffu, hi2 ? v[0] : v[1], 4);
+      v[0] = (hi2 ? v[1] : v[0]) + o;
+      c += hi2 ? 1 : 0;
+      if (R >= 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
+      if (R >= 32) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+    }
+    if (cur.i < a.n) {
+      if (sub < 8 && c < 7) a.out[cur.i * 7 + c] = v[0];
+      if (R == 4 && c + 1 < 7) a.out[cur.i * 7 + c + 1] = v[1];
     }
     cur = nxt;
-    // the next tile's first barrier orders these reads before A2 is rewritten
   }
   cp_async_wait<0>();
   asm volatile("tcgen05.fence::before_thread_sync;");
