@@ -146,24 +146,21 @@ __host__ __device__ constexpr int off(int r, int k, int K) {
   return (r >> 3) * (K / 8) * 128 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
 }
 
-__device__ __forceinline__ uint64_t desc(const void* p, int K) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  uint64_t d = (uint64_t)((a & 0x3FFFF) >> 4);
-  d |= (uint64_t)(128 >> 4) << 16;                 // LBO: next core matrix along K
-  d |= (uint64_t)(((K / 8) * 128) >> 4) << 32;     // SBO: next 8-row group
-  d |= (uint64_t)1 << 46;                           // descriptor version; no swizzle
-  return d;
+// Descriptor of the K-major tile `bytes` after the shared-memory address whose field is
+// `base` (base_of): next core matrix along K 128 bytes on (LBO), next 8-row group K/8 * 128
+// (SBO), descriptor version, no swizzle.  The sum needs no masks or shifts where the MMAs
+// are issued.
+__device__ __forceinline__ uint32_t base_of(const void* p) { return ((uint32_t)__cvta_generic_to_shared(p) & 0x3FFFF) >> 4; }
+__device__ __forceinline__ uint64_t desc_at(uint32_t base, uint32_t bytes, int K) {
+  const uint32_t lo = base + (bytes >> 4) + ((128u >> 4) << 16), hi = (uint32_t)((K / 8) * 128) >> 4 | 1u << 14;
+  return (uint64_t)hi << 32 | lo;
 }
 
 // The same with the 8-row-group stride set to 0: every group of 8 rows reads the same
 // two core matrices, so one 8-row tile stands for a 128-row operand whose rows are
 // all equal.
-__device__ __forceinline__ uint64_t desc_rows_repeated(const void* p) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  uint64_t d = (uint64_t)((a & 0x3FFFF) >> 4);
-  d |= (uint64_t)(128 >> 4) << 16;
-  d |= (uint64_t)1 << 46;
-  return d;
+__device__ __forceinline__ uint64_t desc_rows_repeated(uint32_t base, uint32_t bytes) {
+  return (uint64_t)(1u << 14) << 32 | (base + (bytes >> 4) + ((128u >> 4) << 16));
 }
 
 // kind::f16 instruction descriptor: F32 accumulate, F16 A and B, both K-major.
@@ -288,8 +285,7 @@ __device__ __forceinline__ void stage_fwd_weights(const NeuralDev& nd, unsigned 
 struct Group {                       // one tile in flight
   unsigned char a1[A1_BYTES];
   unsigned char a2[A2_BYTES];          // H1, then the staged output rows
-  uint64_t bar;
-  int abort;
+  uint64_t bar[2];                     // (one used)
 };
 
 struct Smem {
@@ -353,13 +349,68 @@ __device__ __forceinline__ void tc_hidden_tmem(uint32_t taddr) {
   asm volatile("tcgen05.wait::st.sync.aligned;");
 }
 
+// One thread of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// One MMA round trip of a 128-thread group (named barrier 1 + g): what the threads wrote
+// before is visible to the MMAs that issue() starts, and their results to every thread
+// after.  The group's first warp waits for the others, which only arrive, one of its
+// threads issues, and every warp waits on the mbarrier itself.  (Through two barriers and
+// one waiting thread, the waits at the barriers were the decode's largest stall.)
+// A wait that runs out (1.3 s) marks the thread `dead`: it does not wait again, but keeps
+// the barriers' counts, so that the group comes to its end.
+struct Round {
+  uint64_t* bar;
+  uint32_t parity;
+  int g;
+  bool first, dead;
+  template <class Issue>
+  __device__ __forceinline__ void operator()(Issue issue) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (first) {
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (elect_one()) {
+        issue();
+        tc::commit(bar);
+      }
+      __syncwarp();
+    } else {
+      asm volatile("bar.arrive %0, 128;" ::"r"(1 + g) : "memory");
+    }
+    if (!dead) dead = !tc::wait_bar(bar, parity);
+    __syncwarp();
+    parity ^= 1;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+};
+
+__device__ __forceinline__ void fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // Layer 3 from the A operand in columns 0..31: D3 (128 x 16) in columns 32..47, bias included.
-__device__ __forceinline__ void tc_layer3(uint32_t tmem, const unsigned char* b3, const unsigned char* b3x,
-                                          const unsigned char* ones) {
+template <class S>
+__device__ __forceinline__ void tc_layer3(uint32_t tmem, uint32_t sb) {
 #pragma unroll
   for (int kk = 0; kk < 4; ++kk)
-    tc::mma_ts(tmem + 32, tmem + 8 * kk, tc::desc(b3 + kk * 256, 64), tc::idesc(128, 16), kk);
-  tc::mma(tmem + 32, tc::desc_rows_repeated(ones), tc::desc(b3x, 16), tc::idesc(128, 16), 1);
+    tc::mma_ts(tmem + 32, tmem + 8 * kk, tc::desc_at(sb, offsetof(S, b3) + kk * 256, 64), tc::idesc(128, 16), kk);
+  tc::mma(tmem + 32, tc::desc_rows_repeated(sb, offsetof(S, ones)), tc::desc_at(sb, offsetof(S, b3x), 16), tc::idesc(128, 16), 1);
+}
+
+// Layers 1 and 2 from A tiles at a1 and a2 (fields of their addresses): D in columns 0..63.
+template <class S>
+__device__ __forceinline__ void tc_layer1(uint32_t tmem, uint32_t sb, uint32_t a1) {
+  tc::mma(tmem, tc::desc_at(a1, 0, 16), tc::desc_at(sb, offsetof(S, b1), 16), tc::idesc(128, 64), 0);
+}
+template <class S>
+__device__ __forceinline__ void tc_layer2(uint32_t tmem, uint32_t sb, uint32_t a2, int K) {
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk)
+    tc::mma(tmem, tc::desc_at(a2, kk * 256, K), tc::desc_at(sb, offsetof(S, b2) + kk * 256, 64), tc::idesc(128, 64), kk);
+  tc::mma(tmem, tc::desc_rows_repeated(sb, offsetof(S, ones)), tc::desc_at(sb, offsetof(S, b2x), 16), tc::idesc(128, 64), 1);   // + b2
 }
 
 // Named barrier of one 128-thread group.
@@ -380,8 +431,8 @@ template <int F, bool SLIM>
 __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, LookupArgs a) {
   extern __shared__ __align__(1024) unsigned char dyn[];
   tc::Smem& s = *reinterpret_cast<tc::Smem*>(dyn);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int g = tid >> 7, row = tid & 127;          // group, row of the group's tile
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int g = warp >> 2, row = tid & 127;          // group, row of the group's tile
   tc::Group& G = s.grp[g];
   // weights: binary16 images -> K-major no-swizzle B tiles (16-byte rows)
   {
@@ -391,8 +442,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     *reinterpret_cast<uint4*>(G.a1 + tc::off(row, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
   }
   if (row == 0) {
-    G.abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&G.bar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(G.bar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (warp == 0) {
@@ -405,7 +455,8 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = s.tmem + 64 * g;                          // this group's columns
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);  // this warp's lanes
-  uint32_t parity = 0;
+  Round round{G.bar, 0, g, (warp & 3) == 0, false};
+  const uint32_t sb = tc::base_of(&s), a1 = tc::base_of(G.a1), a2 = tc::base_of(G.a2);
   const int64_t ntiles = (a.n + tc::ROWS - 1) / tc::ROWS;
   const int64_t step = 2 * (int64_t)gridDim.x;
   int64_t tile = 2 * (int64_t)blockIdx.x + g;
@@ -419,20 +470,8 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     cp_async_wait<0>();
     uint4 fb = make_uint4(0, 0, 0, 0);
     if (cur.mode == 2) fb = *arow;                   // stored fallback texel (own row)
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    group_sync(g);
-    // layer 1: D[0, 64) = A1 (128 x 16) * W1 (16 x 64); one thread issues and waits
-    if (row == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      tc::mma(tmem, tc::desc(G.a1, 16), tc::desc(s.b1, 16), tc::idesc(128, 64), 0);
-      tc::commit(&G.bar);
-      if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
-    }
-    parity ^= 1;
-    group_sync(g);
-    if (G.abort) break;
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    fence_smem();
+    round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); });
     // A1 is free: start the next tile's gather
     const int64_t next = tile + step;
     NeuralPick nxt;
@@ -440,37 +479,10 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     cp_async_commit();
     qn = load_coords(a, (next + step) * tc::ROWS + row);
     tc_hidden(trow, G.a2, row);
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    group_sync(g);
-    // layer 2: D[0, 64) = H1 (128 x 64) * W2 (64 x 64)
-    if (row == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-        tc::mma(tmem, tc::desc(G.a2 + kk * 256, 64), tc::desc(s.b2 + kk * 256, 64), tc::idesc(128, 64), kk);
-      tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b2x, 16), tc::idesc(128, 64), 1);   // + b2
-      tc::commit(&G.bar);
-      if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
-    }
-    parity ^= 1;
-    group_sync(g);
-    if (G.abort) break;
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    fence_smem();
+    round([&] { tc_layer2<tc::Smem>(tmem, sb, a2, 64); });
     tc_hidden_tmem(trow);
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    group_sync(g);
-    // layer 3: H2 (128 x 64) * W3 (64 x 16)
-    if (row == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      tc_layer3(tmem, s.b3, s.b3x, s.ones);
-      tc::commit(&G.bar);
-      if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
-    }
-    parity ^= 1;
-    group_sync(g);
-    if (G.abort) break;
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    round([&] { tc_layer3<tc::Smem>(tmem, sb); });
     float v[8];
     {
       uint32_t r[8];
@@ -522,7 +534,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
   cp_async_wait<0>();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (row == 0 && G.abort) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
+  if (round.dead) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "n"(tc::TMEM_COLS));
 }
 
@@ -547,7 +559,6 @@ struct Smem {
   unsigned char a2[tc::A2_BYTES];      // H1
   uint64_t bar;
   uint32_t tmem;
-  int abort;
 };
 
 constexpr int TMEM_COLS = 64;
@@ -614,12 +625,11 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
   using Fl = Filter<F>;
   extern __shared__ __align__(1024) unsigned char dyn[];
   tcd::Smem& s = *reinterpret_cast<tcd::Smem*>(dyn);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   tc::stage_fwd_weights(nd, s.b1, s.b2, s.b3, s.b2x, s.b3x, s.ones, tid, 128);
   uint4* arow = reinterpret_cast<uint4*>(s.a1 + tc::off(tid, 0, 16));
   *reinterpret_cast<uint4*>(s.a1 + tc::off(tid, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
   if (tid == 0) {
-    s.abort = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.bar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -633,22 +643,8 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = s.tmem;
   const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
-  uint32_t parity = 0;
-  auto run = [&](auto issue) -> bool {
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      issue();
-      tc::commit(&s.bar);
-      if (!tc::wait_bar(&s.bar, parity)) s.abort = 1;
-    }
-    parity ^= 1;
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    return s.abort == 0;
-  };
+  Round round{&s.bar, 0, 0, warp == 0, false};
+  const uint32_t sb = tc::base_of(&s);
   constexpr int T2 = Fl::T * Fl::T;
   const int parts = (a.lod != nullptr && nd.nlev > 1 && a.level_mode != STF_LEVEL_NEAREST) ? 2 : 1;
   const int R = parts * T2;                    // rows per query: 4, 8, 16 or 32
@@ -666,7 +662,8 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
     uint4 fb = make_uint4(0, 0, 0, 0);
     if (cur.mode == 2) fb = *arow;               // stored fallback texel (own row)
     if (cur.mode != 1) *arow = make_uint4(0, 0, 0, 0);
-    if (!run([&] { tc::mma(tmem, tc::desc(s.a1, 16), tc::desc(s.b1, 16), tc::idesc(128, 64), 0); })) break;
+    fence_smem();
+    round([&] { tc_layer1<tcd::Smem>(tmem, sb, sb + offsetof(tcd::Smem, a1) / 16); });
     // A1 is free: gather the next tile's texels while this tile's layers run
     const int64_t next = tile + gridDim.x;
     DetRow nxt;
@@ -674,14 +671,10 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
     cp_async_commit();
     qn = load_coords(a, (next + gridDim.x) * Q + qi);
     tc_hidden(trow, s.a2, tid);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(s.a2 + kk * 256, 64), tc::desc(s.b2 + kk * 256, 64), tc::idesc(128, 64), kk);
-          tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b2x, 16), tc::idesc(128, 64), 1);
-        }))
-      break;
+    fence_smem();
+    round([&] { tc_layer2<tcd::Smem>(tmem, sb, sb + offsetof(tcd::Smem, a2) / 16, 64); });
     tc_hidden_tmem(trow);
-    if (!run([&] { tc_layer3(tmem, s.b3, s.b3x, s.ones); })) break;
+    round([&] { tc_layer3<tcd::Smem>(tmem, sb); });
     float v[8];
     {
       uint32_t r[8];
@@ -734,7 +727,7 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
   cp_async_wait<0>();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (tid == 0 && s.abort) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
+  if (round.dead) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "n"(tcd::TMEM_COLS));
 }
 
@@ -849,13 +842,11 @@ static_assert(offsetof(Smem, grp) % 128 == 0 && offsetof(Group, h) % 128 == 0, "
 // MN-major operand (no swizzle) from column c0: M or N runs along the columns (core
 // matrices of 8 columns x 8 rows, 128 bytes apart), K along the rows (8-row groups
 // K/8 * 128 bytes apart).  Rows 16 j .. 16 j + 15 start j * K/8 * 256 bytes further.
-__device__ __forceinline__ uint64_t desc_mn(const unsigned char* tile, int c0, int j, int K) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(tile + (c0 >> 3) * 128 + j * (K / 8) * 256);
-  uint64_t d = (uint64_t)((a & 0x3FFFF) >> 4);
-  d |= (uint64_t)(((K / 8) * 128) >> 4) << 16;     // next 8 rows
-  d |= (uint64_t)(128 >> 4) << 32;                 // next 8 columns
-  d |= (uint64_t)1 << 46;
-  return d;
+__device__ __forceinline__ uint64_t desc_mn(uint32_t base, int c0, int j, int K) {
+  const uint32_t lo = base + (((c0 >> 3) * 128 + j * (K / 8) * 256) >> 4) +
+                      ((uint32_t)(((K / 8) * 128) >> 4) << 16);       // next 8 rows
+  const uint32_t hi = (128u >> 4) | 1u << 14;                         // next 8 columns; version
+  return (uint64_t)hi << 32 | lo;
 }
 
 // Both operands MN-major.
@@ -910,8 +901,8 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
   extern __shared__ __align__(1024) unsigned char dyn[];
   tct::Smem& s = *reinterpret_cast<tct::Smem*>(dyn);
   constexpr int NT = 128 * tct::GROUPS;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = tid >> 7, row = tid & 127;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int g = warp >> 2, row = tid & 127;
   tct::Group& G = s.grp[g];
   {
     const uint4* img = reinterpret_cast<const uint4*>(nd.wimg);
@@ -949,24 +940,9 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = s.tmem + tct::COLS * g;
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);   // this warp's lanes
-  uint32_t parity = 0;
-  // make the tiles written so far visible to the tensor cores, let one thread issue
-  // the MMAs, wait for them (bounded), and release the group to read the result
-  auto run = [&](auto issue) -> bool {
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    group_sync(g);
-    if (row == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      issue();
-      tc::commit(&G.bar);
-      if (!tc::wait_bar(&G.bar, parity)) G.abort = 1;
-    }
-    parity ^= 1;
-    group_sync(g);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    return G.abort == 0;
-  };
+  Round round{&G.bar, 0, g, (warp & 3) == 0, false};
+  const uint32_t sb = tc::base_of(&s), gx = tc::base_of(G.x), gdy = tc::base_of(G.dy), gh = tc::base_of(G.h);
+  using S = tct::Smem;
   float sums[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // db3, sum of squared errors
   const int64_t ntiles = (ta.batch + 127) / 128;
   const int64_t step = (int64_t)gridDim.x * tct::GROUPS;
@@ -996,21 +972,21 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     }
     *reinterpret_cast<uint4*>(G.x + tc::off(row, 0, 16)) =
         make_uint4(pack_h2(X[0], X[1]), pack_h2(X[2], X[3]), pack_h2(X[4], X[5]), pack_h2(X[6], X[7]));
-    if (!run([&] { tc::mma(tmem, tc::desc(G.x, 16), tc::desc(s.b1, 16), tc::idesc(128, 64), 0); })) break;
+    fence_smem();
+    round([&] { tc_layer1<S>(tmem, sb, gx); });
     tct_hidden(trow, G.h, 0, row);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(G.h + kk * 256, 128), tc::desc(s.b2 + kk * 256, 64), tc::idesc(128, 64), kk);
-          tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b2x, 16), tc::idesc(128, 64), 1);
-        }))
-      break;
+    fence_smem();
+    round([&] { tc_layer2<S>(tmem, sb, gh, 128); });
     tct_hidden(trow, G.h, 64, row);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(G.h + 1024 + kk * 256, 128), tc::desc(s.b3 + kk * 256, 64), tc::idesc(128, 16), kk);
-          tc::mma(tmem, tc::desc_rows_repeated(s.ones), tc::desc(s.b3x, 16), tc::idesc(128, 16), 1);
-        }))
-      break;
+    fence_smem();
+    round([&] {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc::mma(tmem, tc::desc_at(gh, 1024 + kk * 256, 128), tc::desc_at(sb, offsetof(S, b3) + kk * 256, 64),
+                tc::idesc(128, 16), kk);
+      tc::mma(tmem, tc::desc_rows_repeated(sb, offsetof(S, ones)), tc::desc_at(sb, offsetof(S, b3x), 16),
+              tc::idesc(128, 16), 1);
+    });
     {
       uint32_t y[8];
       tc::tmem_ld<8>(trow, y);
@@ -1032,31 +1008,38 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       }
       *reinterpret_cast<uint4*>(G.dy + tc::off(row, 0, 16)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    if (!run([&] {
-          tc::mma(tmem, tc::desc(G.dy, 16), tc::desc(s.r3, 16), tc::idesc(128, 64), 0);
-          for (int j = 0; j < 8; ++j)
-            tc::mma(tmem + tct::C_W3, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.dy, 0, j, 16),
-                    tct::idesc_mn(128, 16), more | j);
-        }))
-      break;
+    fence_smem();
+    round([&] {
+      tc::mma(tmem, tc::desc_at(gdy, 0, 16), tc::desc_at(sb, offsetof(S, r3), 16), tc::idesc(128, 64), 0);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        tc::mma(tmem + tct::C_W3, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gdy, 0, j, 16), tct::idesc_mn(128, 16),
+                more | j);
+    });
     tct_masked(trow, G.h, 64, row);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(G.h + 1024 + kk * 256, 128), tc::desc(s.r2 + kk * 256, 64), tc::idesc(128, 64), kk);
-          for (int j = 0; j < 8; ++j)
-            tc::mma(tmem + tct::C_W2, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.h, 64, j, 128),
-                    tct::idesc_mn(128, 64), more | j);
-        }))
-      break;
+    fence_smem();
+    round([&] {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc::mma(tmem, tc::desc_at(gh, 1024 + kk * 256, 128), tc::desc_at(sb, offsetof(S, r2) + kk * 256, 64),
+                tc::idesc(128, 64), kk);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        tc::mma(tmem + tct::C_W2, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gh, 64, j, 128), tct::idesc_mn(128, 64),
+                more | j);
+    });
     tct_masked(trow, G.h, 0, row);
-    if (!run([&] {
-          for (int kk = 0; kk < 4; ++kk)
-            tc::mma(tmem, tc::desc(G.h + kk * 256, 128), tc::desc(s.r1 + kk * 256, 64), tc::idesc(128, 16), kk);
-          for (int j = 0; j < 8; ++j)
-            tc::mma(tmem + tct::C_W1, tct::desc_mn(G.h, 0, j, 128), tct::desc_mn(G.x, 0, j, 16),
-                    tct::idesc_mn(128, 16), more | j);
-        }))
-      break;
+    fence_smem();
+    round([&] {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc::mma(tmem, tc::desc_at(gh, kk * 256, 128), tc::desc_at(sb, offsetof(S, r1) + kk * 256, 64),
+                tc::idesc(128, 16), kk);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        tc::mma(tmem + tct::C_W1, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gx, 0, j, 16), tct::idesc_mn(128, 16),
+                more | j);
+    });
     more = 1;
     float dx[8];
     {
@@ -1100,10 +1083,11 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     if (lane == 0) s.sums[warp][k] = sums[k];
   }
   if (row == 0) G.tiles = (int)more;
+  if (round.dead) G.abort = 1;
   float* stage = reinterpret_cast<float*>(G.h);       // dW2 64 x 64, then dW3 or dW1 and db 9 x 128
   const bool upper = row >= 64;
   uint32_t v[32];
-  if (g > 0 && more && G.abort == 0) {
+  if (g > 0 && more) {
 #pragma unroll
     for (int cb = 0; cb < 2; ++cb) {
       tc::tmem_ld<32>(trow + tct::C_W2 + 32 * cb, v);
