@@ -370,6 +370,11 @@ struct Round {
   bool first, dead;
   template <class Issue>
   __device__ __forceinline__ void operator()(Issue issue) {
+    start(issue);
+    finish();
+  }
+  template <class Issue>
+  __device__ __forceinline__ void start(Issue issue) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (first) {
       asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
@@ -382,6 +387,8 @@ struct Round {
     } else {
       asm volatile("bar.arrive %0, 128;" ::"r"(1 + g) : "memory");
     }
+  }
+  __device__ __forceinline__ void finish() {
     if (!dead) dead = !tc::wait_bar(bar, parity);
     __syncwarp();
     parity ^= 1;
@@ -472,15 +479,16 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     if (cur.mode == 2) fb = *arow;                   // stored fallback texel (own row)
     fence_smem();
     round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); });
-    // A1 is free: start the next tile's gather
+    tc_hidden(trow, G.a2, row);
+    fence_smem();
+    round.start([&] { tc_layer2<tc::Smem>(tmem, sb, a2, 64); });
+    // while layer 2 runs (A1 is free): the next tile's tap choices and gather
     const int64_t next = tile + step;
     NeuralPick nxt;
     if (next < ntiles) nxt = neural_pick<F, SLIM>(nd, a, next * tc::ROWS + row, arow, &qn);
     cp_async_commit();
     qn = load_coords(a, (next + step) * tc::ROWS + row);
-    tc_hidden(trow, G.a2, row);
-    fence_smem();
-    round([&] { tc_layer2<tc::Smem>(tmem, sb, a2, 64); });
+    round.finish();
     tc_hidden_tmem(trow);
     round([&] { tc_layer3<tc::Smem>(tmem, sb); });
     float v[8];
@@ -664,15 +672,16 @@ __global__ void __launch_bounds__(128, 6) k_neural_deterministic_tc(NeuralDev nd
     if (cur.mode != 1) *arow = make_uint4(0, 0, 0, 0);
     fence_smem();
     round([&] { tc_layer1<tcd::Smem>(tmem, sb, sb + offsetof(tcd::Smem, a1) / 16); });
-    // A1 is free: gather the next tile's texels while this tile's layers run
+    tc_hidden(trow, s.a2, tid);
+    fence_smem();
+    round.start([&] { tc_layer2<tcd::Smem>(tmem, sb, sb + offsetof(tcd::Smem, a2) / 16, 64); });
+    // while layer 2 runs (A1 is free): the next tile's taps and gather
     const int64_t next = tile + gridDim.x;
     DetRow nxt;
     if (next < ntiles) nxt = det_row<F>(nd, a, next * Q + qi, p, tx, ty, arow, &qn);
     cp_async_commit();
     qn = load_coords(a, (next + gridDim.x) * Q + qi);
-    tc_hidden(trow, s.a2, tid);
-    fence_smem();
-    round([&] { tc_layer2<tcd::Smem>(tmem, sb, sb + offsetof(tcd::Smem, a2) / 16, 64); });
+    round.finish();
     tc_hidden_tmem(trow);
     round([&] { tc_layer3<tcd::Smem>(tmem, sb); });
     float v[8];
