@@ -15,7 +15,6 @@
 // returns sum(w t) / sum(w).  Every step of the tap decision is a float32 operation
 // in a fixed order (no contraction), so any float32 implementation of the same steps
 // makes the same choice.
-#include <climits>
 #include <cmath>
 #include <cstring>
 
@@ -89,9 +88,9 @@ struct Ellipse {
 __device__ __forceinline__ Ellipse ewa_ellipse(const Footprint& f, float2 uv, float WL, float HL) {
   float d0u = __fmul_rn(f.Mx, WL), d0v = __fmul_rn(f.My, HL);
   float d1u = __fmul_rn(f.mx, WL), d1v = __fmul_rn(f.my, HL);
-  const float m = __fsqrt_rn(__fadd_rn(__fmul_rn(d1u, d1u), __fmul_rn(d1v, d1v)));
-  if (m > 2.0f) {
-    const float k = __fdiv_rn(2.0f, m);
+  const float m2 = __fadd_rn(__fmul_rn(d1u, d1u), __fmul_rn(d1v, d1v));
+  if (m2 > 0x1.000002p+2f) {          // the square root rounds to more than 2
+    const float k = __fdiv_rn(2.0f, __fsqrt_rn(m2));
     d0u = __fmul_rn(d0u, k);
     d0v = __fmul_rn(d0v, k);
     d1u = __fmul_rn(d1u, k);
@@ -102,12 +101,12 @@ __device__ __forceinline__ Ellipse ewa_ellipse(const Footprint& f, float2 uv, fl
   float B = __fmul_rn(-2.0f, __fadd_rn(__fmul_rn(d0u, d0v), __fmul_rn(d1u, d1v)));
   float C = __fadd_rn(__fadd_rn(__fmul_rn(d0u, d0u), __fmul_rn(d1u, d1u)), 1.0f);
   const float F = __fsub_rn(__fmul_rn(A, C), __fmul_rn(__fmul_rn(B, B), 0.25f));
-  const float inv = __fdiv_rn(1.0f, F);
+  const float inv = __frcp_rn(F);
   A = __fmul_rn(A, inv);
   B = __fmul_rn(B, inv);
   C = __fmul_rn(C, inv);
   const float det = __fsub_rn(__fmul_rn(__fmul_rn(4.0f, A), C), __fmul_rn(B, B));
-  const float inv_det = __fdiv_rn(1.0f, det);
+  const float inv_det = __frcp_rn(det);
   const float hs = __fmul_rn(__fmul_rn(2.0f, inv_det), __fsqrt_rn(__fmul_rn(det, C)));
   const float ht = __fmul_rn(__fmul_rn(2.0f, inv_det), __fsqrt_rn(__fmul_rn(A, det)));
   e.A = A;
@@ -151,6 +150,175 @@ __device__ __forceinline__ float ewa_weight(const Ellipse& e, const float* lut, 
   return lut[max((int)__fmul_rn(r2, (float)kEwaLut), 0)];
 }
 
+// The weights of texels is and is + 1 (x = their float coordinates) of a row: the same
+// operations and roundings as ewa_weight, for an ellipse with ewa_plain().  The second
+// texel may lie past the box's end, where its weight is 0 without a test: the box ends
+// where Q reaches 1, to a relative error far below 1/128, and the table's last entry
+// (Q from 127/128) is exactly 0.  Float counters
+// replace the integer conversions, the last addition saturates (Q < 0 counts as 0; Q >= 1
+// becomes 1, whose entry lut[128] is 0), and adding 2^23 rounding towards zero leaves the
+// table index in the low mantissa bits.  9 issued instructions a texel, against 14 with
+// conversions and a test: the loops over texels bound both
+// forms (5.4 M queries of a 4K ground plane: 130 -> 107 us stochastic, 153 -> 133 us
+// deterministic).
+__device__ __forceinline__ float ewa_lut_at(uint32_t lut, float r2x128) {
+  // (no volatile: the table does not change after it was staged)
+  float w;
+  asm("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(lut + (__float_as_uint(r2x128) << 2)));
+  return w;
+}
+
+__device__ __forceinline__ float sat_add(float a, float b) {
+  float r;
+  asm("add.rn.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+__device__ __forceinline__ float2 ewa_weight2(const Ellipse& e, uint32_t lut, float2 x, const EwaRow& row) {
+  // (packed additions only: a packed multiplication and the addition after it are
+  // contracted into a multiply-add, which moved a table index now and then)
+  const float2 ss = __fadd2_rn(x, make_float2(-e.st_s, -e.st_s));
+  const float s0 = ss.x, s1 = ss.y;
+  const float r0 = sat_add(__fmul_rn(__fadd_rn(__fmul_rn(e.A, s0), row.Btt), s0), row.Ctt2);
+  const float r1 = sat_add(__fmul_rn(__fadd_rn(__fmul_rn(e.A, s1), row.Btt), s1), row.Ctt2);
+  return make_float2(ewa_lut_at(lut, __fmaf_rz(r0, (float)kEwaLut, 8388608.0f)),
+                     ewa_lut_at(lut, __fmaf_rz(r1, (float)kEwaLut, 8388608.0f)));
+}
+
+// Shared-memory address of the table, less the offset that 2^23's bits add (modulo 2^32).
+__device__ __forceinline__ uint32_t ewa_lut_base(const float* lut) {
+  return (uint32_t)__cvta_generic_to_shared(lut) - (0x4B000000u << 2);
+}
+
+// Finite coefficients, and coordinates that count up exactly in float32.  Other ellipses
+// (derivatives near the float32 range, uv beyond 2^23 texels) take the checked loops.
+__device__ __forceinline__ bool ewa_plain(const Ellipse& e) {
+  return fabsf(e.st_s) < 8380000.0f && fabsf(e.st_t) < 8380000.0f && fabsf(e.A) <= 3.4e38f && fabsf(e.B) <= 3.4e38f &&
+         fabsf(e.C) <= 3.4e38f;
+}
+
+struct EwaLevel {
+  int64_t off;
+  int32_t w, h;
+};
+
+// Texel (cx, cy) of level L, already clamped to it.
+template <int FMT, int C>
+__device__ __forceinline__ void ewa_texel(const Tex2DView& t, int L, const EwaLevel& lv, int cx, int cy, float* v) {
+  if constexpr (FMT == STF_FMT_DCT6) dct_texel<C>(t, L, cx, cy, v);
+  else TexelIO<FMT, C>::load(t.texels, lv.off + (int64_t)cy * lv.w + cx, v);
+}
+
+// Inverse-CDF choice over the box's texels in row-major order.  Pass 1: the running
+// float32 sum, recorded at the end of each of the first kEwaRows rows.  Pass 2 resumes
+// from the last recorded value below u S, so it rescans one row in the common case and
+// repeats exactly the same additions.  (Adding a zero weight leaves a float32 sum
+// unchanged, so texels outside the ellipse are summed without a test.)
+template <bool PLAIN>
+__device__ __forceinline__ bool ewa_choose(const Ellipse& e, const float* lut, float u, int& cs, int& ct) {
+  const uint32_t base = ewa_lut_base(lut);
+  const float x0 = (float)e.s0, x1 = (float)e.s1;
+  float S = 0.0f;
+  float row_end[kEwaRows];
+  for (int it = e.t0; it <= e.t1; ++it) {
+    const EwaRow row = ewa_row(e, it);
+    if constexpr (PLAIN) {
+      for (float2 x = make_float2(x0, x0 + 1.0f); x.x <= x1; x = __fadd2_rn(x, make_float2(2.0f, 2.0f))) {
+        const float2 w = ewa_weight2(e, base, x, row);
+        S = __fadd_rn(__fadd_rn(S, w.x), w.y);
+      }
+    } else {
+      for (int is = e.s0; is <= e.s1; ++is) S = __fadd_rn(S, ewa_weight(e, lut, is, row));
+    }
+    if (it - e.t0 < kEwaRows) row_end[it - e.t0] = S;
+  }
+  const float us = __fmul_rn(u, S);
+  float Cs = 0.0f;
+  int start = e.t0;
+  const int cached = min(e.t1 - e.t0 + 1, kEwaRows);
+  for (int k = 0; k < cached && row_end[k] <= us; ++k) {
+    Cs = row_end[k];
+    start = e.t0 + k + 1;
+  }
+  // (us < C_k is never first true right after a zero weight)
+  for (int it = start; it <= e.t1; ++it) {
+    const EwaRow row = ewa_row(e, it);
+    ct = it;
+    if constexpr (PLAIN) {
+      for (float2 x = make_float2(x0, x0 + 1.0f); x.x <= x1; x = __fadd2_rn(x, make_float2(2.0f, 2.0f))) {
+        const float2 w = ewa_weight2(e, base, x, row);
+        const float C1 = __fadd_rn(Cs, w.x);
+        Cs = __fadd_rn(C1, w.y);
+        if (us < Cs) {
+          cs = (int)(us < C1 ? x.x : x.y);
+          return true;
+        }
+      }
+    } else {
+      for (cs = e.s0; cs <= e.s1; ++cs) {
+        Cs = __fadd_rn(Cs, ewa_weight(e, lut, cs, row));
+        if (us < Cs) return true;
+      }
+    }
+  }
+  return false;
+}
+
+// Sum of the weights, and of weight times texel per channel.
+template <int FMT, int C, bool PLAIN>
+__device__ __forceinline__ float ewa_average(const Tex2DView& t, int L, const EwaLevel& lv, const Ellipse& e,
+                                             const float* lut, float* acc) {
+  const uint32_t base = ewa_lut_base(lut);
+  const float x0 = (float)e.s0;
+  float S = 0.0f;
+#pragma unroll
+  for (int c = 0; c < C; ++c) acc[c] = 0.0f;
+  auto texel = [&](int is, int cy, float* tv) {
+    ewa_texel<FMT, C>(t, L, lv, min(max(is, 0), lv.w - 1), cy, tv);
+  };
+  for (int it = e.t0; it <= e.t1; ++it) {
+    const EwaRow row = ewa_row(e, it);
+    const int cy = min(max(it, 0), lv.h - 1);
+    if constexpr (PLAIN) {
+      float2 x = make_float2(x0, x0 + 1.0f);
+      for (int is = e.s0; is <= e.s1; is += 2) {
+        const float2 w = ewa_weight2(e, base, x, row);
+        x = __fadd2_rn(x, make_float2(2.0f, 2.0f));
+        float ta[C], tb[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) ta[c] = tb[c] = 0.0f;
+        if (w.x > 0.0f) texel(is, cy, ta);
+        if (w.y > 0.0f) texel(is + 1, cy, tb);
+        S = __fadd_rn(__fadd_rn(S, w.x), w.y);
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c] = fmaf(w.y, tb[c], fmaf(w.x, ta[c], acc[c]));
+      }
+    } else {
+      for (int is = e.s0; is <= e.s1; ++is) {
+        const float w = ewa_weight(e, lut, is, row);
+        if (w > 0.0f) {
+          float tv[C];
+          texel(is, cy, tv);
+          S = __fadd_rn(S, w);
+#pragma unroll
+          for (int c = 0; c < C; ++c) acc[c] = fmaf(w, tv[c], acc[c]);
+        }
+      }
+    }
+  }
+  return S;
+}
+
+// The checked loops, out of the way.
+__device__ __noinline__ bool ewa_choose_checked(Ellipse e, const float* lut, float u, int* cs, int* ct) {
+  return ewa_choose<false>(e, lut, u, *cs, *ct);
+}
+template <int FMT, int C>
+__device__ __noinline__ float ewa_average_checked(const Tex2DView* t, int L, EwaLevel lv, Ellipse e, const float* lut,
+                                                  float* acc) {
+  return ewa_average<FMT, C, false>(*t, L, lv, e, lut, acc);
+}
+
 struct EwaArgs {
   const float* uv;      // n x 2
   const float4* grad;   // n x (du/dx, dv/dx, du/dy, dv/dy)
@@ -168,14 +336,17 @@ struct EwaArgs {
 
 // Per query: stochastic (one texel) or deterministic (weighted average, two levels
 // blended by frac(lod) in the stochastic level mode).
+// At most kFastLoopMaxQueries queries.
 template <int FMT, int C, bool STOCH>
 __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable tab) {
-  __shared__ float lut[kEwaLut];
-  for (int k = threadIdx.x; k < kEwaLut; k += blockDim.x) lut[k] = tab.w[k];
+  __shared__ float lut[kEwaLut + 1];                  // and the weight 0 of Q >= 1
+  __shared__ EwaLevel levels[STF_MAX_LEVELS];         // (lanes index it apart)
+  if (threadIdx.x < t.levels) levels[threadIdx.x] = {t.level_off[threadIdx.x], t.level_w[threadIdx.x], t.level_h[threadIdx.x]};
+  for (int k = threadIdx.x; k <= kEwaLut; k += blockDim.x) lut[k] = k < kEwaLut ? tab.w[k] : 0.0f;
   __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
   const float W0 = (float)t.level_w[0], H0 = (float)t.level_h[0];
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const float2 uv = reinterpret_cast<const float2*>(a.uv)[i];
     const float4 g = a.grad[i];
     float v[C];
@@ -183,8 +354,8 @@ __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable ta
     for (int c = 0; c < C; ++c) v[c] = 0.0f;
     int4 tap = make_int4(0, 0, 0, -1);
     const Footprint f = ewa_footprint(g, W0, H0, a.max_aniso);
-    const bool finite_in = isfinite(uv.x) && isfinite(uv.y) && isfinite(g.x) && isfinite(g.y) &&
-                           isfinite(g.z) && isfinite(g.w) && f.ok;
+    // (finite squared lengths imply finite derivatives)
+    const bool finite_in = isfinite(uv.x) && isfinite(uv.y) && f.ok;
     if (finite_in) {
       const float lc = fminf(fmaxf(f.lod, 0.0f), (float)(t.levels - 1));
       int L0, L1 = 0;
@@ -195,48 +366,28 @@ __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable ta
                                       a.key0, a.key1);
         const float u_level = a.level_mode == STF_LEVEL_NEAREST ? 0.5f : unit24(r.w);
         L0 = t.levels <= 1 ? 0 : min((int)floorf(__fadd_rn(lc, u_level)), t.levels - 1);
-        const int WL = t.level_w[L0], HL = t.level_h[L0];
+        const EwaLevel lv = levels[L0];
+        const int WL = lv.w, HL = lv.h;
         const Ellipse e = ewa_ellipse(f, uv, (float)WL, (float)HL);
         if (!ewa_span_ok(e)) {
           atomicOr(a.status, STF_DEV_BAD_NODE);
         } else {
-          // Pass 1: the running float32 sum, recorded at the end of each of the first
-          // kEwaRows rows.  Pass 2 resumes from the last recorded value below u S, so it
-          // rescans one row in the common case and repeats exactly the same additions.
-          float S = 0.0f;
-          float row_end[kEwaRows];
-          // (adding a zero weight leaves a float32 sum unchanged, so texels outside
-          // the ellipse are summed without a test)
-          for (int it = e.t0; it <= e.t1; ++it) {
-            const EwaRow row = ewa_row(e, it);
-            for (int is = e.s0; is <= e.s1; ++is) S = __fadd_rn(S, ewa_weight(e, lut, is, row));
-            if (it - e.t0 < kEwaRows) row_end[it - e.t0] = S;
+          int cs = 0, ct = 0;
+          const float u = unit24(r.x);
+          bool found;
+          if (ewa_plain(e)) {
+            found = ewa_choose<true>(e, lut, u, cs, ct);
+          } else {
+            int s2 = 0, t2 = 0;
+            found = ewa_choose_checked(e, lut, u, &s2, &t2);
+            cs = s2;
+            ct = t2;
           }
-          const float us = __fmul_rn(unit24(r.x), S);
-          float Cs = 0.0f;
-          int start = e.t0;
-          const int cached = min(e.t1 - e.t0 + 1, kEwaRows);
-          for (int k = 0; k < cached && row_end[k] <= us; ++k) {
-            Cs = row_end[k];
-            start = e.t0 + k + 1;
-          }
-          int cs = INT_MIN, ct = 0;
-          for (int it = start; it <= e.t1 && cs == INT_MIN; ++it) {
-            const EwaRow row = ewa_row(e, it);
-            for (int is = e.s0; is <= e.s1; ++is) {
-              Cs = __fadd_rn(Cs, ewa_weight(e, lut, is, row));
-              if (us < Cs) {   // never true right after a zero weight
-                cs = is;
-                ct = it;
-                break;
-              }
-            }
-          }
-          if (cs == INT_MIN) {
+          if (!found) {
             atomicOr(a.status, STF_DEV_BAD_NODE);   // cannot happen: us < S
           } else {
             tap = make_int4(cs, ct, 0, L0);
-            fetch2d<FMT, C>(t, L0, min(max(cs, 0), WL - 1), min(max(ct, 0), HL - 1), v);
+            ewa_texel<FMT, C>(t, L0, lv, min(max(cs, 0), WL - 1), min(max(ct, 0), HL - 1), v);
           }
         }
       } else {
@@ -252,28 +403,21 @@ __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable ta
         for (int part = 0; part < (frac > 0.0f ? 2 : 1); ++part) {
           const int L = part ? L1 : L0;
           const float wl = part ? frac : 1.0f - frac;
-          const int WL = t.level_w[L], HL = t.level_h[L];
+          const EwaLevel lv = levels[L];
+          const int WL = lv.w, HL = lv.h;
           const Ellipse e = ewa_ellipse(f, uv, (float)WL, (float)HL);
           if (!ewa_span_ok(e)) {
             atomicOr(a.status, STF_DEV_BAD_NODE);
             continue;
           }
-          float S = 0.0f, acc[C];
+          float acc[C], S;
+          if (ewa_plain(e)) {
+            S = ewa_average<FMT, C, true>(t, L, lv, e, lut, acc);
+          } else {
+            float a2[C];
+            S = ewa_average_checked<FMT, C>(&t, L, lv, e, lut, a2);
 #pragma unroll
-          for (int c = 0; c < C; ++c) acc[c] = 0.0f;
-          for (int it = e.t0; it <= e.t1; ++it) {
-            const EwaRow row = ewa_row(e, it);
-            const int cy = min(max(it, 0), HL - 1);
-            for (int is = e.s0; is <= e.s1; ++is) {
-              const float w = ewa_weight(e, lut, is, row);
-              if (w > 0.0f) {
-                float tv[C];
-                fetch2d<FMT, C>(t, L, min(max(is, 0), WL - 1), cy, tv);
-                S = __fadd_rn(S, w);
-#pragma unroll
-                for (int c = 0; c < C; ++c) acc[c] = fmaf(w, tv[c], acc[c]);
-              }
-            }
+            for (int c = 0; c < C; ++c) acc[c] = a2[c];
           }
           const float k = __fdiv_rn(wl, S);
 #pragma unroll
@@ -298,9 +442,19 @@ __global__ void k_aniso_lod(EwaArgs a, float W0, float H0, int levels) {
 
 template <int FMT, int C>
 static cudaError_t run_ewa(bool stoch, const Tex2DView& t, const EwaArgs& a, cudaStream_t s) {
-  const int blocks = grid_blocks(a.n, 256);
-  if (stoch) k_ewa<FMT, C, true><<<blocks, 256, 0, s>>>(t, a, ewa_table());
-  else k_ewa<FMT, C, false><<<blocks, 256, 0, s>>>(t, a, ewa_table());
+  // slices of 32-bit indices
+  for (int64_t i = 0; i < a.n; i += kFastLoopMaxQueries) {
+    EwaArgs b = a;
+    b.uv += 2 * i;
+    b.grad += i;
+    b.out += C * i;
+    if (b.taps) b.taps += 4 * i;
+    b.query_offset += (uint64_t)i;
+    b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
+    const int blocks = grid_blocks(b.n, 256);
+    if (stoch) k_ewa<FMT, C, true><<<blocks, 256, 0, s>>>(t, b, ewa_table());
+    else k_ewa<FMT, C, false><<<blocks, 256, 0, s>>>(t, b, ewa_table());
+  }
   return cudaGetLastError();
 }
 

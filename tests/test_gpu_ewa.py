@@ -212,3 +212,22 @@ def test_full_size_ewa_plane_sampled():
     gv = out.cpu().numpy()[idx].astype(np.float64)
     assert np.array_equal(gv[same], rv[same])
     stf.stf_synchronize(T.handle)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1000.0, 1.4e5])
+def test_ewa_far_coordinates_match_oracle(scale):
+    """Coordinates up to beyond 2^23 texels, where the fast texel loops give way to the
+    checked ones, and boxes of odd and even widths: taps and averages against the oracle."""
+    T, ref = _texture()
+    uv, g = _queries(1500, 64, 11)
+    uv = (uv * np.float32(scale)).astype(np.float32)
+    taps = torch.empty((len(uv), 4), dtype=torch.int32, device=dev())
+    T.lookup_ewa(to_dev(uv), to_dev(g), 16.0, taps=taps, seed=17)
+    _, rt, ex = ewa.lookup(ref, uv, g, 16.0, stochastic_form=True, seed=17)
+    same = np.all(taps.cpu().numpy() == rt, axis=1)
+    assert np.all(same | ex)
+    det = T.lookup_ewa_deterministic(to_dev(uv), to_dev(g), 16.0).cpu().numpy().astype(np.float64)
+    dv, _, tol = ewa.lookup(ref, uv, g, 16.0, stochastic_form=False)
+    ok = np.isfinite(tol)
+    assert np.all(np.abs(det - dv)[ok] <= (2e-6 * np.abs(dv) + tol[:, None])[ok])
+    stf.stf_synchronize(T.handle)
