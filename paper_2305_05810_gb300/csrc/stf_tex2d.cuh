@@ -171,6 +171,37 @@ __device__ __forceinline__ void tex2d_det_at(const Tex2DView& t, const LookupArg
   }
 }
 
+// Levels of a deterministic lookup and their weights: one level (nearest mode or no lod)
+// or floor(lod) and the next blended by frac(lod); weights 0 for a lod that is not finite.
+struct DetLevels {
+  int L0, L1;
+  float w0, w1;
+};
+
+__device__ __forceinline__ DetLevels det_levels(const Tex2DView& t, const LookupArgs& a, float lod) {
+  DetLevels d = {0, 0, isfinite(lod) ? 1.0f : 0.0f, 0.0f};
+  if (a.lod == nullptr || t.levels <= 1 || d.w0 == 0.0f) return d;
+  const float lc = fminf(fmaxf(lod, 0.0f), (float)(t.levels - 1));
+  if (a.level_mode == STF_LEVEL_NEAREST) {
+    d.L0 = min((int)floorf(__fadd_rn(lc, 0.5f)), t.levels - 1);
+  } else {
+    const float fl = floorf(lc);
+    d.w1 = __fsub_rn(lc, fl);
+    d.w0 = 1.0f - d.w1;
+    d.L0 = (int)fl;
+    d.L1 = min(d.L0 + 1, t.levels - 1);
+  }
+  return d;
+}
+
+// The same at uv.
+template <int F, int FMT, int C>
+__device__ __forceinline__ void tex2d_det_uv(const Tex2DView& t, int L, float2 uv, float scale, float width, float* acc) {
+  float x[2] = {__fsub_rn(__fmul_rn(uv.x, (float)t.level_w[L]), 0.5f),
+                __fsub_rn(__fmul_rn(uv.y, (float)t.level_h[L]), 0.5f)};
+  if (prepare_coords<2>(x)) tex2d_det_level<F, FMT, C>(t, L, x, scale, width, acc);
+}
+
 // ---------------------------------------------------------------- triplanar
 
 struct Planes {
@@ -265,28 +296,16 @@ __device__ __forceinline__ void dct_det_warp(const Tex2DView& t, const LookupArg
                                              float2 uv, float lod, float scale, const float2* basis, DctItems& items,
                                              float* acc) {
   const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
-  int L[2] = {0, 0};
-  float part[2] = {1.0f, 0.0f};
-  ok = ok && isfinite(lod);
-  if (ok && a.lod != nullptr && t.levels > 1) {
-    const float lc = fminf(fmaxf(lod, 0.0f), (float)(t.levels - 1));
-    if (a.level_mode == STF_LEVEL_NEAREST) {
-      L[0] = min((int)floorf(__fadd_rn(lc, 0.5f)), t.levels - 1);
-    } else {
-      const float fl = floorf(lc);
-      part[1] = __fsub_rn(lc, fl);
-      part[0] = 1.0f - part[1];
-      L[0] = (int)fl;
-      L[1] = min(L[0] + 1, t.levels - 1);
-    }
-  }
+  const DetLevels d = det_levels(t, a, lod);
+  const int L[2] = {d.L0, d.L1};
+  const float part[2] = {d.w0, d.w1};
   uint32_t first[2] = {0, 0}, count[2] = {0, 0}, total = 0;
 #pragma unroll
   for (int p = 0; p < 2; ++p) {
     if (p == 1 && !__any_sync(0xffffffffu, ok && part[1] > 0.0f)) break;
     const DctLevel lv = levels[L[p]];
     float x[2] = {__fsub_rn(__fmul_rn(uv.x, (float)lv.w), 0.5f), __fsub_rn(__fmul_rn(uv.y, (float)lv.h), 0.5f)};
-    const bool on = ok && (p == 0 || part[1] > 0.0f) && prepare_coords<2>(x);
+    const bool on = ok && part[p] > 0.0f && prepare_coords<2>(x);
     if (!on) x[0] = x[1] = 0.0f;
     DctAxis<F> ax(x[0], lv.w, t.dct_k[0], basis), ay(x[1], lv.h, t.dct_k[0], basis);
     const float sc = scale * part[p];
@@ -436,10 +455,57 @@ __global__ void __launch_bounds__(256) k_tex2d_stochastic(Tex2DView t, LookupArg
   }
 }
 
+// ---------------------------------------------------------------- deterministic, scattered warps
+//
+// The cubic filters of plain textures.  With one thread per query, the 16 loads of a warp
+// whose queries lie apart each read 32 lines, and the L1 data pipe bounds the filter (96%
+// busy).  Such a warp runs its queries in four rounds of eight instead, four lanes to a
+// query, one per tap column: the lanes read the four neighbouring texels of a row in one
+// load, and their partial sums meet by halving exchanges.  A warp whose queries are
+// neighbours shares lines between lanes already and keeps one thread per query, which
+// sets up its weights once instead of four times.  4.2 M random lookups of a 256^2 FP32
+// RGBA texture: 168 -> 103 us; in raster order unchanged (54 us; 94 us by columns).
+
+// Raster position of a query at level L, and whether it takes part.
+struct RasterPos {
+  float x[2];
+  int L;
+  bool on;
+  __device__ __forceinline__ RasterPos(const Tex2DView& t, int L_, float2 uv, bool ok) : L(L_) {
+    x[0] = __fsub_rn(__fmul_rn(uv.x, (float)t.level_w[L]), 0.5f);
+    x[1] = __fsub_rn(__fmul_rn(uv.y, (float)t.level_h[L]), 0.5f);
+    on = ok && prepare_coords<2>(x);
+  }
+};
+
+// Column k of the window at raster position (x, y) of level L, weighted by `scale`, added
+// to acc.
 template <int F, int FMT, int C>
-__global__ void __launch_bounds__(256) k_tex2d_deterministic(Tex2DView t, LookupArgs a) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+__device__ __forceinline__ void tex2d_det_column(const Tex2DView& t, int L, float x, float y, float scale, int k,
+                                                 float* acc) {
+  using Fl = Filter<F>;
+  const int W = t.level_w[L], H = t.level_h[L];
+  float fx, fy, wx[4], wy[4];
+  const int bx = axis_base(x, fx) + Fl::OFF0, by = axis_base(y, fy) + Fl::OFF0;
+  Fl::weights(fx, wx);
+  Fl::weights(fy, wy);
+  const float wk = k == 0 ? wx[0] : k == 1 ? wx[1] : k == 2 ? wx[2] : wx[3];
+  const int cx = min(max(bx + k, 0), W - 1);
+#pragma unroll
+  for (int ky = 0; ky < 4; ++ky) {
+    float tv[C];
+    fetch2d<FMT, C>(t, L, cx, min(max(by + ky, 0), H - 1), tv);
+    const float w = wk * (wy[ky] * scale);
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = fmaf(w, tv[c], acc[c]);
+  }
+}
+
+// One thread per query: the loop of the filters that do not gather by warp.
+template <int F, int FMT, int C, typename I>
+__device__ __forceinline__ void tex2d_det_loop(const Tex2DView& t, const LookupArgs& a) {
+  const I n = (I)a.n, stride = (I)gridDim.x * blockDim.x;
+  for (I i = (I)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const float2 uv = reinterpret_cast<const float2*>(a.coords)[i];
     const float lod = a.lod ? a.lod[i] : 0.0f;
     float acc[C];
@@ -448,6 +514,91 @@ __global__ void __launch_bounds__(256) k_tex2d_deterministic(Tex2DView t, Lookup
     tex2d_det_at<F, FMT, C>(t, a, uv, lod, 1.0f, acc);
     store_out<C>(a.out, i, acc);
   }
+}
+
+// At most kFastLoopMaxQueries queries; a warp's first ones decide how it takes all of its
+// queries.  With levels of detail
+// only texels of 16 bytes and more gain (8-channel FP16 122 us against 136, 4-channel FP16
+// 105 against 90 for 2.1 M queries at random levels: the second level's setup is paid
+// four times as well).
+template <int F, int FMT, int C>
+__global__ void __launch_bounds__(256) k_tex2d_cubic(Tex2DView t, LookupArgs a) {
+  constexpr uint32_t full = 0xffffffffu;
+  const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+  const int lane = threadIdx.x & 31, k = lane & 3;
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x;
+  if (C * (FMT == STF_FMT_F32 ? 4 : 2) < 16 && a.lod != nullptr && t.levels > 1) {
+    tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
+    return;
+  }
+  {
+    // lanes whose neighbour's level-0 window is within a few texels of theirs
+    const float2 uv = first < n ? reinterpret_cast<const float2*>(a.coords)[first] : make_float2(0.0f, 0.0f);
+    const float x = uv.x * (float)t.level_w[0], y = uv.y * (float)t.level_h[0];
+    const float dx = __shfl_xor_sync(full, x, 1) - x, dy = __shfl_xor_sync(full, y, 1) - y;
+    if (__popc(__ballot_sync(full, fabsf(dx) < 5.0f && fabsf(dy) < 2.0f)) >= 16) {
+      tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
+      return;
+    }
+  }
+  // (every lane of a warp runs the same iterations)
+  for (uint32_t i0 = first - lane; i0 < n; i0 += stride) {
+    const uint32_t i = i0 + lane;
+    const bool live = i < n;
+    const float2 uv = live ? reinterpret_cast<const float2*>(a.coords)[i] : make_float2(0.0f, 0.0f);
+    const float lod = live && a.lod ? a.lod[i] : 0.0f;
+    const DetLevels d = det_levels(t, a, lod);
+    const RasterPos p(t, d.L0, uv, live && d.w0 > 0.0f);
+    const RasterPos p1(t, d.L1, uv, live && d.w1 > 0.0f);
+    const bool blend = __any_sync(full, p1.on);
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {
+      const int src = 8 * r + (lane >> 2);
+      float v[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) v[c] = 0.0f;
+      {
+        const float x = __shfl_sync(full, p.x[0], src), y = __shfl_sync(full, p.x[1], src);
+        const float sc = __shfl_sync(full, d.w0, src);
+        const int L = __shfl_sync(full, p.on ? p.L : -1, src);
+        if (L >= 0) tex2d_det_column<F, FMT, C>(t, L, x, y, sc, k, v);
+      }
+      if (blend) {
+        const float x = __shfl_sync(full, p1.x[0], src), y = __shfl_sync(full, p1.x[1], src);
+        const float sc = __shfl_sync(full, d.w1, src);
+        const int L = __shfl_sync(full, p1.on ? p1.L : -1, src);
+        if (L >= 0) tex2d_det_column<F, FMT, C>(t, L, x, y, sc, k, v);
+      }
+      // sum over the four lanes; each exchange halves the channels a lane keeps
+      int c0 = 0;
+#pragma unroll
+      for (int off = 2, kept = C; off >= 1; off /= 2) {
+        const bool up = k & off;
+        if (kept > 1) {
+          kept /= 2;
+#pragma unroll
+          for (int c = 0; c < kept; ++c) {
+            const float o = __shfl_xor_sync(full, up ? v[c] : v[c + kept], off);
+            v[c] = (up ? v[c + kept] : v[c]) + o;
+          }
+          c0 += up ? kept : 0;
+        } else {
+          v[0] += __shfl_xor_sync(full, v[0], off);
+        }
+      }
+      const uint32_t j = i0 + src;
+      if (j < n && (C >= 4 || (C == 2 && !(k & 1)) || k == 0)) {
+        float* o = a.out + (size_t)j * C + c0;
+        if constexpr (C == 8) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+        else *o = v[0];
+      }
+    }
+  }
+}
+
+template <int F, int FMT, int C>
+__global__ void __launch_bounds__(256) k_tex2d_deterministic(Tex2DView t, LookupArgs a) {
+  tex2d_det_loop<F, FMT, C, int64_t>(t, a);
 }
 
 template <int F, int FMT, int C, bool REUSE>
@@ -554,6 +705,16 @@ static cudaError_t run_tex2d(Op op, const Tex2DView& t, const LookupArgs& a, cud
     }
   } else if (op == OP_DETERMINISTIC) {
     if constexpr (DctByBlock<D, FMT>::value) k_dct_deterministic<D, C, false><<<grid_blocks(a.n, 128), 128, 0, s>>>(t, a);
+    else if constexpr (FMT != STF_FMT_DCT6 && (D == STF_FILTER_BSPLINE3 || D == STF_FILTER_CATMULL_ROM)) {
+      for (int64_t i = 0; i < a.n; i += kFastLoopMaxQueries) {        // slices of 32-bit indices
+        LookupArgs b = a;
+        b.coords += 2 * i;
+        if (b.lod) b.lod += i;
+        b.out += C * i;
+        b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
+        k_tex2d_cubic<D, FMT, C><<<grid_blocks(b.n, threads), threads, 0, s>>>(t, b);
+      }
+    }
     else k_tex2d_deterministic<D, FMT, C><<<blocks, threads, 0, s>>>(t, a);
   } else {
     if constexpr (UsesReuse<F>::value) {

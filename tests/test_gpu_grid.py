@@ -443,3 +443,33 @@ def test_degenerate_sizes(filt):
         det = T.lookup_deterministic(to_dev(pts), filter=filt)
         dv, _, _ = filters.lookup_3d(ref, pts, filt, stochastic_form=False)
         check_deterministic(det.cpu().numpy(), dv, 2.0)
+
+
+@pytest.mark.parametrize("channels", [1, 2, 4, 8])
+@pytest.mark.parametrize("fmt", [stf.FMT_F32, stf.FMT_F16])
+def test_cubic_scattered_and_neighbouring_warps(fmt, channels):
+    """The cubic deterministic filters take a warp of scattered queries four lanes to a
+    query and a warp of neighbours one lane to a query: both against the oracle, in one call
+    that mixes them with invalid queries and ends in a part of a warp, without levels of
+    detail and with two levels blended."""
+    W, H, levels = 64, 32, 4
+    base = synth.texture2d(W, H, channels, seed=5)
+    T = stf.Texture(stf.KIND_TEX2D, base, dims=(W, H, 1), channels=channels, mip_levels=levels,
+                    generate_mips=True, fmt=fmt)
+    ref = textures.Texture2D([quantise(l, fmt) for l in synth.box_levels(base, levels)])
+    n = 1024 + 13
+    uv = synth.uv_queries(n, seed=6) * np.float32(1.2) - np.float32(0.1)
+    row = np.arange(512, dtype=np.float32)
+    uv[256:768, 0], uv[256:768, 1] = (row % 64) / 64 + 1 / 128, (row // 64) / 16
+    uv[5], uv[300, 0], uv[n - 1, 1] = np.nan, np.inf, 3e7
+    lod = synth.lods(n, seed=7, lo=-0.5, hi=3.5)
+    lod[256:512] = 0.0
+    lod[9] = np.nan
+    for filt in ("bspline3", "catmull_rom"):
+        for l in (None, lod):
+            det = T.lookup_deterministic(to_dev(uv), None if l is None else to_dev(l), filter=filt).cpu().numpy()
+            dv, _, _ = filters.lookup_2d(ref, uv, l, filt, stochastic_form=False)
+            # texels in [0, 1], |weights| sum to at most 1.25 per axis; the generated mips are
+            # float32 means, within 2^-23 of the oracle's (and one binary16 rounding step)
+            lim = 2e-6 * 1.25 ** 2 + (2.0 ** -11 if fmt == stf.FMT_F16 and l is not None else 0.0)
+            assert np.all(np.abs(det - dv) <= lim)
