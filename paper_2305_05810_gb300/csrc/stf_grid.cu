@@ -254,11 +254,13 @@ __global__ void __launch_bounds__(256, dense_stochastic_min_blocks<F>()) k_dense
   }
 }
 
-// The T consecutive voxels e .. e + T - 1 of one grid row.  FP16 rows of four come from
-// the aligned 16 bytes (eight voxels) that hold e, plus the next 8 bytes when the row
-// runs over (e mod 8 > 4), shifted into place; the texel allocation is padded by 16 bytes,
-// so neither leaves it.  (Two aligned 8-byte words, needed for 3 of 4 rows, took 15% more
-// load wavefronts at the same time.)  Other rows are read voxel by voxel.
+// The T consecutive voxels e .. e + T - 1 of one grid row, from the aligned word that holds
+// e plus, when the row runs over it, the start of the next one: 16 bytes (eight FP16
+// voxels, and 8 bytes more for e mod 8 > 4; four FP32 voxels, and 16 bytes more for
+// e mod 4 > 0) for rows of four, two voxels (and one more for odd e) for rows of two.  The
+// texel allocation is padded by 16 bytes, so no load leaves it.  The L1 wavefronts of these
+// loads bound the filters.  (Two aligned 8-byte words for FP16 rows of four, needed for 3
+// of 4 rows, took 15% more of them at the same time.)
 template <int FMT, int T>
 __device__ __forceinline__ void dense_row(const void* texels, uint32_t e, float* v) {
   if constexpr (FMT == STF_FMT_F16 && T == 4) {
@@ -274,13 +276,34 @@ __device__ __forceinline__ void dense_row(const void* texels, uint32_t e, float*
     const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&lo));
     const float2 f1 = __half22float2(*reinterpret_cast<const __half2*>(&hi));
     v[0] = f0.x; v[1] = f0.y; v[2] = f1.x; v[3] = f1.y;
+  } else if constexpr (FMT == STF_FMT_F32 && T == 4) {
+    const float4* w = reinterpret_cast<const float4*>(texels) + (e >> 2);
+    const float4 a = __ldg(w);
+    float4 b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (e & 3) b = __ldg(w + 1);
+    const bool by2 = e & 2, by1 = e & 1;
+    const float y0 = by2 ? a.z : a.x, y1 = by2 ? a.w : a.y, y2 = by2 ? b.x : a.z, y3 = by2 ? b.y : a.w,
+                y4 = by2 ? b.z : b.x;
+    v[0] = by1 ? y1 : y0; v[1] = by1 ? y2 : y1; v[2] = by1 ? y3 : y2; v[3] = by1 ? y4 : y3;
+  } else if constexpr (FMT == STF_FMT_F16) {
+    static_assert(T == 2, "rows of two or four");
+    const __half2 a = __ldg(reinterpret_cast<const __half2*>(texels) + (e >> 1));
+    v[0] = __high2float(a);
+    if (e & 1) {
+      v[1] = __half2float(__ldg(reinterpret_cast<const __half*>(texels) + e + 1));
+    } else {
+      v[1] = v[0];
+      v[0] = __low2float(a);
+    }
   } else {
-#pragma unroll
-    for (int k = 0; k < T; ++k) {
-      if constexpr (FMT == STF_FMT_F16)
-        v[k] = __half2float(__ldg(reinterpret_cast<const __half*>(texels) + e + k));
-      else
-        v[k] = __ldg(reinterpret_cast<const float*>(texels) + e + k);
+    static_assert(T == 2, "rows of two or four");
+    const float2 a = __ldg(reinterpret_cast<const float2*>(texels) + (e >> 1));
+    v[0] = a.y;
+    if (e & 1) {
+      v[1] = __ldg(reinterpret_cast<const float*>(texels) + e + 1);
+    } else {
+      v[1] = v[0];
+      v[0] = a.x;
     }
   }
 }
