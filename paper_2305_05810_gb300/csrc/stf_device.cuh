@@ -351,7 +351,7 @@ struct LookupArgs {
 // tests (3 i + 2 then stays below 2^32); other calls take the general 64-bit loop.
 constexpr int64_t kFastLoopMaxQueries = int64_t(1) << 30;
 
-__device__ __forceinline__ bool fast_loop(const LookupArgs& a) {
+__host__ __device__ __forceinline__ bool fast_loop(const LookupArgs& a) {
   return a.perm == nullptr && a.taps == nullptr && a.n <= kFastLoopMaxQueries;
 }
 
@@ -447,6 +447,58 @@ __device__ __forceinline__ void load_and_clear(const LookupArgs& a, float backgr
       for (int d = 0; d < 3; ++d) x[k][d] = __ldg(a.coords + 3 * (i0 + k) + d);
       a.out[i0 + k] = background;
     }
+  }
+}
+
+// The stochastic lookups of a filter with a fixed window, by queue.  Each warp walks
+// chunks of 32 * PER queries, writes the background and keeps those whose window reaches
+// into `live` in shared memory (at most 31 and a chunk); whenever 32 wait, work(i, x, ok)
+// draws and fetches one per lane.  The next chunk's coordinates load meanwhile.
+template <int PER>
+struct LiveQueue {
+  static constexpr int CAP = 32 * (PER + 1);
+  uint32_t i[CAP];
+  float x[3][CAP];
+};
+
+template <int PER, class Work>
+__device__ __forceinline__ void live_queue_loop(const LookupArgs& a, float background, const LiveBox& live,
+                                                LiveQueue<PER>& q, Work work) {
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u, n = (uint32_t)a.n;
+  const bool aligned = (((uintptr_t)a.coords | (uintptr_t)a.out) & 15) == 0;
+  uint32_t waiting = 0;
+  WarpChunks<32 * PER> w;
+  float x[PER][3];
+  load_and_clear<PER>(a, background, aligned, w.first() + lane * PER, n, x);
+  for (;;) {
+    const bool more = w.row < n;                     // else: only what still waits
+    const uint32_t i0 = w.first() + lane * PER;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const bool in = live.has(x[k]);
+      const uint32_t m = __ballot_sync(0xffffffffu, in);
+      if (in) {
+        const uint32_t s = waiting + __popc(m & below);
+        q.i[s] = i0 + k;
+        q.x[0][s] = x[k][0]; q.x[1][s] = x[k][1]; q.x[2][s] = x[k][2];
+      }
+      waiting += __popc(m);
+    }
+    w.next();
+    load_and_clear<PER>(a, background, aligned, w.first() + lane * PER, n, x);
+    __syncwarp();          // the queue and the background stores, before other lanes' results
+    while (waiting >= (more ? 32u : 1u)) {
+      const uint32_t count = min(waiting, 32u);
+      waiting -= count;
+      const bool ok = lane < count;
+      const uint32_t s = waiting + lane;
+      float y[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) y[d] = ok ? q.x[d][s] : 0.0f;
+      work(ok ? q.i[s] : 0u, y, ok);
+    }
+    if (!more) break;
+    __syncwarp();          // the slots just read may be filled again
   }
 }
 
@@ -596,15 +648,13 @@ __device__ __forceinline__ void pick_fis(const float* x, const LookupArgs& a, in
   }
 }
 
-// Filters whose dense 3D stochastic lookups take the joint four-query form: one tap
-// from one set of draws per query, independent variates per axis, and a gain measured
-// on the dense benchmark rays (tent +14%, B-spline +6%, FIS tent +8%, FIS B-spline +5%,
-// FIS Gaussian +3%).  Catmull-Rom measured 4% slower in it and keeps the one-query
-// form; so do the two-tap positivized estimator and the sparse grids, whose traversal
-// per tap measured 7% slower joint.
+// Filters whose dense 3D stochastic lookups take the joint four-query form: the Gaussian
+// (3% sooner than one query after another on the dense benchmark rays).  The fixed-window
+// filters go by queue; Catmull-Rom measured 4% slower in it and keeps the one-query form,
+// as do the two-tap positivized estimator and the sparse grids (7% slower).
 template <int F, bool REUSE>
 struct JointOneTap {
-  static constexpr bool value = (F == STF_FILTER_LINEAR || F == STF_FILTER_BSPLINE3 || IsFis<F>::value) && !REUSE;
+  static constexpr bool value = F == STF_FILTER_FIS_GAUSSIAN && !REUSE;
 };
 
 // The tap of one such lookup at coordinates x (checked by prepare_coords) from its

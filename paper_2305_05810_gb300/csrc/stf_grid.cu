@@ -82,115 +82,32 @@ __device__ __forceinline__ float dense_stochastic_one(const Dense3DView& g, cons
   return dense_stochastic_at<F, FMT, REUSE, OFF32>(g, a, x, j, sample, tap);
 }
 
-// Packed form of the four-query loop for the fixed-window filters (tent, B-spline, and
-// their FIS forms): a warp's 128 queries are tested against the miss box, each lane
-// writes the background over its four results, and the warp's live queries are then
-// packed onto its lanes, lane t taking the live queries of rank t, t + 32, ... in
-// (query-in-group, lane) order, R = ceil(live / 32) per lane, drawn, chosen and gathered
-// side by side.  A warp with at most 64 live queries thus runs one or two draws per lane
-// instead of four; a warp with more keeps each lane's own four (joint_one_tap4).  The
-// packed lanes reload their queries' coordinates (from L1: the warp has just read them)
-// and store each result over the background its owner wrote.
-// Position of the set bit of rank n (0-based) in m, for n < popc(m): a binary search on
-// the population counts of the low halves.
-__device__ __forceinline__ uint32_t nth_set_bit(uint32_t m, uint32_t n) {
-  uint32_t pos = 0;
-#pragma unroll
-  for (int w = 16; w >= 1; w >>= 1) {
-    const uint32_t low = __popc(m & ((1u << w) - 1u));
-    if (n >= low) {
-      n -= low;
-      m >>= w;
-      pos += (uint32_t)w;
-    }
+// Stochastic lookups of the fixed-window filters (tent, B-spline and their FIS forms), of
+// grids of at most 2^32 voxels and at most kFastLoopMaxQueries queries, without tap output
+// or permutation.  A ray-march chunk holds from none to three quarters of live samples; the
+// queue lets every draw run on full lanes.  33 M samples of a 256^3 FP16 grid, B-spline:
+// 133 us with the live ones of each chunk packed on its own lanes (two or four draws a
+// lane), 117 us by queue (88 M instead of 117 M warp instructions; the coordinates kept
+// beside the indices instead of read again: 4 us; the next chunk loaded ahead on five
+// blocks an SM instead of six: 3 us; two draws a lane: 3 us slower).
+constexpr int kDenseQueueBlocks = 5;      // resident 256-thread blocks per SM
+template <int F, int FMT, int PER>
+__global__ void __launch_bounds__(256, kDenseQueueBlocks) k_dense_stochastic_queue(Dense3DView g, LookupArgs a) {
+  using W = FixedWindow<F>;
+  __shared__ LiveQueue<PER> queues[8];
+  __shared__ LiveBox live;
+  if (threadIdx.x == 0) {
+    const int zero[3] = {0, 0, 0}, dims[3] = {g.nx, g.ny, g.nz};
+    live = live_box(zero, dims, W::LO, W::HI);
   }
-  return pos;
-}
-
-template <int F, int FMT, int R>
-__device__ __forceinline__ void dense_packed_rounds(const Dense3DView& g, const LookupArgs& a, uint32_t q0,
-                                                    const uint32_t (&b)[4], uint32_t live_count, uint32_t lane,
-                                                    uint32_t groups) {
-  const uint32_t c0 = __popc(b[0]), c1 = c0 + __popc(b[1]), c2 = c1 + __popc(b[2]);
-  uint32_t qi[R];
-  bool ok[R];
-  float x[R][3];
-#pragma unroll
-  for (int q = 0; q < R; ++q) {
-    const uint32_t r = lane + 32u * (uint32_t)q;
-    ok[q] = r < live_count;
-    const int k = r < c0 ? 0 : r < c1 ? 1 : r < c2 ? 2 : 3;
-    const uint32_t before = k == 0 ? 0u : k == 1 ? c0 : k == 2 ? c1 : c2;
-    const uint32_t bk = k == 0 ? b[0] : k == 1 ? b[1] : k == 2 ? b[2] : b[3];
-    const uint32_t src = ok[q] ? nth_set_bit(bk, r - before) : 0u;
-    qi[q] = 4u * (q0 + src) + (uint32_t)k;
-    ok[q] = ok[q] && qi[q] < 4u * groups;    // a live query lies in an active lane's group
-    x[q][0] = x[q][1] = x[q][2] = 0.0f;
-    if (ok[q]) {
-      x[q][0] = __ldg(a.coords + 3 * qi[q]);
-      x[q][1] = __ldg(a.coords + 3 * qi[q] + 1);
-      x[q][2] = __ldg(a.coords + 3 * qi[q] + 2);
-    }
-    prepare_coords<3>(x[q]);            // the owner's clamp of huge coordinates, again
-  }
-  uint4 rv[R];
-#pragma unroll
-  for (int q = 0; q < R; ++q) rv[q] = query_variates(a, qi[q], a.sample_index);
-  int t[R][3];
-#pragma unroll
-  for (int q = 0; q < R; ++q) draw_one_tap3<F>(a, x[q], qi[q], rv[q], t[q]);
-#pragma unroll
-  for (int q = 0; q < R; ++q)
-    if (ok[q]) a.out[qi[q]] = dense_fetch<FMT, true>(g, t[q][0], t[q][1], t[q][2]);
-}
-
-template <int F, int FMT>
-__device__ __forceinline__ void dense_packed_loop(const Dense3DView& g, const LookupArgs& a, const MissBox& mb) {
-  const uint32_t n = (uint32_t)a.n, groups = n >> 2, stride = gridDim.x * blockDim.x;
-  const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31u;
-  const float4* c4 = reinterpret_cast<const float4*>(a.coords);
-  float4* o4 = reinterpret_cast<float4*>(a.out);
-  const float bg = g.background;
-  // every lane of a warp runs the same iterations (the loop bound is the warp's first
-  // group), so the warp-wide votes below see all 32 lanes
-  for (uint32_t w0 = tid - lane; w0 < groups; w0 += stride) {
-    const uint32_t gq = w0 + lane;
-    const bool act = gq < groups;
-    float x[4][3] = {};
-    bool live[4] = {false, false, false, false};
-    if (act) {
-      const float4 p = __ldg(c4 + 3 * gq), q = __ldg(c4 + 3 * gq + 1), r = __ldg(c4 + 3 * gq + 2);
-      x[0][0] = p.x; x[0][1] = p.y; x[0][2] = p.z;
-      x[1][0] = p.w; x[1][1] = q.x; x[1][2] = q.y;
-      x[2][0] = q.z; x[2][1] = q.w; x[2][2] = r.x;
-      x[3][0] = r.y; x[3][1] = r.z; x[3][2] = r.w;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) live[k] = prepare_coords<3>(x[k]) && !misses(mb, x[k]);
-    }
-    uint32_t b[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) b[k] = __ballot_sync(0xffffffffu, live[k]);
-    const uint32_t live_count = __popc(b[0]) + __popc(b[1]) + __popc(b[2]) + __popc(b[3]);
-    // (every branch below is the same for all lanes)
-    if (live_count > 64) {
-      // mostly live: each lane its own four queries, side by side
-      if (act) o4[gq] = joint_one_tap4<F>(a, x, 4 * gq, mb, bg, [&](const int* t) {
-        return dense_fetch<FMT, true>(g, t[0], t[1], t[2]);
-      });
-      continue;
-    }
-    if (act) o4[gq] = make_float4(bg, bg, bg, bg);
-    if (live_count == 0) continue;
-    __syncwarp();                        // the owners' background stores come first
-    if (live_count <= 32) dense_packed_rounds<F, FMT, 1>(g, a, w0, b, live_count, lane, groups);
-    else dense_packed_rounds<F, FMT, 2>(g, a, w0, b, live_count, lane, groups);
-    __syncwarp();
-  }
-  for (uint32_t i = 4 * groups + tid; i < n; i += stride) {
-    float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
-    int4 tap;
-    a.out[i] = dense_stochastic_at<F, FMT, false, true>(g, a, x, i, a.sample_index, tap, &mb);
-  }
+  __syncthreads();
+  live_queue_loop<PER>(a, g.background, live, queues[threadIdx.x >> 5], [&](uint32_t i, float (&x)[3], bool ok) {
+    const uint4 v = query_variates(a, i, a.sample_index);
+    prepare_coords<3>(x);
+    int t[3];
+    draw_one_tap3<F>(a, x, i, v, t);
+    if (ok) a.out[i] = dense_fetch<FMT, true>(g, t[0], t[1], t[2]);
+  });
 }
 
 // Resident 256-thread blocks per SM: six (at most 40 registers a thread) for the tent
@@ -209,12 +126,6 @@ __global__ void __launch_bounds__(256, dense_stochastic_min_blocks<F>()) k_dense
                                                                                          LookupArgs a) {
   const bool off32 = (uint64_t)g.nx * (uint64_t)g.ny * (uint64_t)g.nz <= (uint64_t(1) << 32);
   const MissBox mb = miss_box<F>(0, 0, 0, g.nx, g.ny, g.nz);
-  if constexpr (FixedWindow<F>::value && F != STF_FILTER_FIS_BSPLINE3 && !REUSE) {
-    if (off32 && quad_loop3_ok(a)) {
-      dense_packed_loop<F, FMT>(g, a, mb);
-      return;
-    }
-  }
   if constexpr (JointOneTap<F, REUSE>::value) {
     if (off32 && quad_loop3_ok(a)) {
       quad_loop3_joint(a, [&](float (&x)[4][3], uint32_t i) {
@@ -228,22 +139,24 @@ __global__ void __launch_bounds__(256, dense_stochastic_min_blocks<F>()) k_dense
       return;
     }
   }
-  if (off32 && quad_loop3_ok(a)) {
-    quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
-      float x[3] = {x0, x1, x2};
-      int4 tap;
-      return dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, j, a.sample_index, tap, &mb);
-    });
-    return;
-  }
-  if (fast_loop(a) && off32) {
-    const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-      float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
-      int4 tap;
-      a.out[i] = dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, i, a.sample_index, tap, &mb);
+  if constexpr (!FixedWindow<F>::value || REUSE) {   // (the others went by queue)
+    if (off32 && quad_loop3_ok(a)) {
+      quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
+        float x[3] = {x0, x1, x2};
+        int4 tap;
+        return dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, j, a.sample_index, tap, &mb);
+      });
+      return;
     }
-    return;
+    if (fast_loop(a) && off32) {
+      const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
+        int4 tap;
+        a.out[i] = dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, i, a.sample_index, tap, &mb);
+      }
+      return;
+    }
   }
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
@@ -495,6 +408,16 @@ static cudaError_t run_dense(Op op, const Dense3DView& g, const LookupArgs& a, c
   const int64_t units = (op == OP_STOCHASTIC && quad_loop3_ok(a)) ? (a.n + 3) / 4 : a.n;
   const int blocks = grid_blocks(units, threads, op == OP_STOCHASTIC ? kStochasticWaves : 4);
   if (op == OP_STOCHASTIC) {
+    if constexpr (FixedWindow<F>::value) {
+      const bool off32 = (uint64_t)g.nx * (uint64_t)g.ny * (uint64_t)g.nz <= (uint64_t(1) << 32);
+      if (off32 && fast_loop(a) && !(UsesReuse<F>::value && a.reuse)) {
+        if (a.n >= kQueueChunkMin)
+          k_dense_stochastic_queue<F, FMT, 4><<<queue_blocks((a.n + 3) / 4, threads, kDenseQueueBlocks), threads, 0, s>>>(g, a);
+        else
+          k_dense_stochastic_queue<F, FMT, 1><<<queue_blocks(a.n, threads, kDenseQueueBlocks), threads, 0, s>>>(g, a);
+        return cudaGetLastError();
+      }
+    }
     if constexpr (UsesReuse<F>::value) {
       if (a.reuse) k_dense_stochastic<F, FMT, true><<<blocks, threads, 0, s>>>(g, a);
       else k_dense_stochastic<F, FMT, false><<<blocks, threads, 0, s>>>(g, a);

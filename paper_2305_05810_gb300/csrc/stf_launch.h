@@ -21,7 +21,7 @@ int queue_blocks(int64_t n, int threads, int per_sm);
 // 3% slower at 5.3M with 16).
 constexpr int kStochasticWaves = 8;
 
-// Deterministic 3D calls of at least this many queries take chunks of 128 per warp (three
+// Queued 3D calls of at least this many queries take chunks of 128 per warp (three
 // 16-byte coordinate loads per lane, fuller queues); below it chunks of 32 spread a
 // call over more warps.
 constexpr int64_t kQueueChunkMin = 1 << 20;

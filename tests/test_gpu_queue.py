@@ -131,3 +131,26 @@ def test_sparse_neighbours_of_non_finite_voxels_are_not_read():
     touched = np.all((base >= 3) & (base <= 6), axis=1)
     assert np.array_equal(a[~touched], b[~touched])
     assert np.isnan(b[touched]).all() and touched.any()
+
+
+@pytest.mark.parametrize("filt", ["linear", "bspline3", "fis_linear", "fis_bspline3"])
+@pytest.mark.parametrize("kind", ["dense", "sparse"])
+def test_stochastic_queue_equals_the_general_loop(kind, filt):
+    """Queued stochastic calls (chunks of 32 and of 128; aligned and misaligned arrays; ragged
+    ends; few, most and no queries live; counters that cross 2^32) against the call with tap
+    output, which takes the general loop."""
+    T, _ = _dense(stf.FMT_F16) if kind == "dense" else _sparse(stf.FMT_E4M3_SCALED)
+    for n, spread in ((1, 1.0), (33, 1.0), (4099, 1.0), (CHUNKED + 77, 1.0), (CHUNKED + 77, 0.01), (CHUNKED, 100.0)):
+        p = _points(n, 0, 23, 5) if kind == "dense" else _points(n, -32, 32, 5)
+        p = p * np.float32(spread)
+        p = (p + (np.float32(8) if kind == "dense" else np.array([128, 0, 4096], np.float32))).astype(np.float32)
+        for shift in (0, 1):
+            buf = torch.empty((n + 1, 3), dtype=torch.float32, device=dev())
+            c = buf[shift:shift + n]
+            c.copy_(to_dev(p))
+            out = torch.full((n + 1, 1), 7.0, device=dev())
+            args = dict(filter=filt, seed=11, query_offset=(1 << 32) - 1000)
+            T.lookup(c, out=out[shift:shift + n], **args)
+            want = T.lookup(c, taps=torch.empty((n, 4), dtype=torch.int32, device=dev()), **args)
+            torch.testing.assert_close(out[shift:shift + n], want, rtol=0, atol=0)
+            assert float(out[0 if shift else n]) == 7.0
