@@ -884,6 +884,39 @@ __device__ __forceinline__ void tct_masked(uint32_t taddr, unsigned char* h, int
   }
 }
 
+// One texel of a training batch: its latents and target (zeros past the end).
+struct TrainRow {
+  int64_t id, epoch;
+  float x[8], t[7];
+  bool live;
+  __device__ __forceinline__ void load(const NeuralDev& nd, const TrainArgs& ta, int64_t r) {
+    live = r < ta.batch;
+    id = epoch = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) t[k] = 0.0f;
+    if (!live) return;
+    if (ta.ids) {
+      id = ta.ids[r];
+    } else {
+      const int64_t gp = ta.step * ta.batch + r;
+      epoch = gp / nd.n_lat_texels;
+      id = permute_index(gp % nd.n_lat_texels, nd.n_lat_texels, ta.seed);
+    }
+    const float4 x0 = reinterpret_cast<const float4*>(nd.lat32 + id * 8)[0];
+    const float4 x1 = reinterpret_cast<const float4*>(nd.lat32 + id * 8)[1];
+    x[0] = x0.x; x[1] = x0.y; x[2] = x0.z; x[3] = x0.w;
+    x[4] = x1.x; x[5] = x1.y; x[6] = x1.z; x[7] = x1.w;
+    const float* tp = ta.target_rows ? ta.target_rows + r * 7 : ta.target_levels + id * 7;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) t[k] = tp[k];
+  }
+};
+
+// A tile's texels are gathered ahead of its turn: the first one's before the weights are
+// staged, the next one's during the backward round trips (a batch's texels are distinct, so
+// the latents' update in between does not touch them).
 __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(NeuralDev nd, TrainArgs ta) {
   extern __shared__ __align__(1024) unsigned char dyn[];
   tct::Smem& s = *reinterpret_cast<tct::Smem*>(dyn);
@@ -891,6 +924,11 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int g = warp >> 2, row = tid & 127;
   tct::Group& G = s.grp[g];
+  const int64_t ntiles = (ta.batch + 127) / 128;
+  const int64_t step = (int64_t)gridDim.x * tct::GROUPS;
+  int64_t tile = blockIdx.x + (int64_t)gridDim.x * g;
+  TrainRow cur;
+  cur.load(nd, ta, tile * 128 + row);
   {
     const uint4* img = reinterpret_cast<const uint4*>(nd.wimg);
     const uint4 z = make_uint4(0, 0, 0, 0);
@@ -931,32 +969,11 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
   const uint32_t sb = tc::base_of(&s), gx = tc::base_of(G.x), gdy = tc::base_of(G.dy), gh = tc::base_of(G.h);
   using S = tct::Smem;
   float sums[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // db3, sum of squared errors
-  const int64_t ntiles = (ta.batch + 127) / 128;
-  const int64_t step = (int64_t)gridDim.x * tct::GROUPS;
-  int64_t tile = blockIdx.x + (int64_t)gridDim.x * g;
   uint32_t more = 0;                          // 0 for the group's first tile: accumulators start from zero
   for (; tile < ntiles; tile += step) {
     const int64_t r = tile * 128 + row;
-    const bool live = r < ta.batch;
-    int64_t id = 0, epoch = 0;
-    float T[7] = {0, 0, 0, 0, 0, 0, 0};
-    float X[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (live) {
-      if (ta.ids) {
-        id = ta.ids[r];
-      } else {
-        const int64_t gp = ta.step * ta.batch + r;
-        epoch = gp / nd.n_lat_texels;
-        id = permute_index(gp % nd.n_lat_texels, nd.n_lat_texels, ta.seed);
-      }
-      const float4 x0 = reinterpret_cast<const float4*>(nd.lat32 + id * 8)[0];
-      const float4 x1 = reinterpret_cast<const float4*>(nd.lat32 + id * 8)[1];
-      X[0] = x0.x; X[1] = x0.y; X[2] = x0.z; X[3] = x0.w;
-      X[4] = x1.x; X[5] = x1.y; X[6] = x1.z; X[7] = x1.w;
-      const float* tp = ta.target_rows ? ta.target_rows + r * 7 : ta.target_levels + id * 7;
-#pragma unroll
-      for (int k = 0; k < 7; ++k) T[k] = tp[k];
-    }
+    const bool live = cur.live;
+    const float* X = cur.x;
     *reinterpret_cast<uint4*>(G.x + tc::off(row, 0, 16)) =
         make_uint4(pack_h2(X[0], X[1]), pack_h2(X[2], X[3]), pack_h2(X[4], X[5]), pack_h2(X[6], X[7]));
     fence_smem();
@@ -980,7 +997,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       float d[8];
 #pragma unroll
       for (int k = 0; k < 7; ++k) {
-        const float e = live ? __uint_as_float(y[k]) - T[k] : 0.0f;
+        const float e = live ? __uint_as_float(y[k]) - cur.t[k] : 0.0f;
         sums[7] = fmaf(e, e, sums[7]);
         d[k] = 2.0f * ta.inv_batch * e;
       }
@@ -995,6 +1012,8 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       }
       *reinterpret_cast<uint4*>(G.dy + tc::off(row, 0, 16)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
+    TrainRow nxt;
+    nxt.load(nd, ta, (tile + step) * 128 + row);
     fence_smem();
     round([&] {
       tc::mma(tmem, tc::desc_at(gdy, 0, 16), tc::desc_at(sb, offsetof(S, r3), 16), tc::idesc(128, 64), 0);
@@ -1042,12 +1061,12 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       }
       if (ta.train) {
         // Adam on this latent row; its update count is its epoch + 1 (one visit per epoch)
-        const float tt = (float)(epoch + 1);
+        const float tt = (float)(cur.epoch + 1);
         const float c1 = 1.0f - powf(ta.beta1, tt), c2 = 1.0f - powf(ta.beta2, tt);
         float xn[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int64_t e = id * 8 + k;
+          const int64_t e = cur.id * 8 + k;
           const float mm = ta.beta1 * nd.m_lat[e] + (1.0f - ta.beta1) * dx[k];
           const float vv = ta.beta2 * nd.v_lat[e] + (1.0f - ta.beta2) * dx[k] * dx[k];
           nd.m_lat[e] = mm;
@@ -1055,11 +1074,12 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
           xn[k] = X[k] - ta.lr * (mm / c1) / (sqrtf(vv / c2) + ta.eps);
           nd.lat32[e] = xn[k];
         }
-        reinterpret_cast<uint4*>(const_cast<__half*>(nd.lat16))[id] =
+        reinterpret_cast<uint4*>(const_cast<__half*>(nd.lat16))[cur.id] =
             make_uint4(pack_h2(xn[0], xn[1]), pack_h2(xn[2], xn[3]), pack_h2(xn[4], xn[5]),
                        pack_h2(xn[6], xn[7]));
       }
     }
+    cur = nxt;
   }
   // The groups' gradients: groups 1 and 2 leave their rows in their own tiles, [column]
   // [row], group 0 adds them to its own and takes them to memory.
