@@ -259,3 +259,20 @@ def test_gradients_by_batch_size(batch):
     stf.stf_neural_gradients(T.handle, i, batch, t, None, None, loss)
     assert abs(loss.item() - want) <= 2e-3 * want
     stf.stf_synchronize(T.handle)
+
+
+def test_gradients_into_page_locked_memory():
+    """Parameter gradients and loss into page-locked host memory: float32 sums in another
+    order of the same products as the ones on the device, 1e-4 of the norm apart at most."""
+    T, ref, lat, par, pyr = make_neural(size=32, latent_levels=3, levels=3)
+    rng = np.random.default_rng(4)
+    i = to_dev(rng.integers(0, lat.shape[0], 1000).astype(np.int64))
+    t = to_dev(rng.standard_normal((1000, 7)).astype(np.float32))
+    n = stf.NEURAL_PARAMS
+    pg, loss = torch.empty(n, device=dev()), torch.empty(1, device=dev())
+    hg, hl = torch.zeros(n, pin_memory=True), torch.zeros(1, pin_memory=True)
+    stf.stf_neural_gradients(T.handle, i, 1000, t, pg, None, loss)
+    stf.stf_neural_gradients(T.handle, i, 1000, t, hg, None, hl)
+    assert (hg - pg.cpu()).norm() <= 1e-4 * pg.norm().item()
+    assert abs(hl.item() - loss.item()) <= 1e-4 * loss.item()
+    stf.stf_synchronize(T.handle)
