@@ -15,6 +15,7 @@
 #include <math.h>
 
 #include "stf_internal.h"
+#include "stf_round.h"
 
 namespace stf {
 
@@ -285,7 +286,8 @@ __device__ __forceinline__ void stage_fwd_weights(const NeuralDev& nd, unsigned 
 struct Group {                       // one tile in flight
   unsigned char a1[A1_BYTES];
   unsigned char a2[A2_BYTES];          // H1, then the staged output rows
-  uint64_t bar[2];                     // (one used)
+  uint64_t bar;
+  uint64_t pad;
 };
 
 struct Smem {
@@ -356,45 +358,26 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// One MMA round trip of a 128-thread group (named barrier 1 + g): what the threads wrote
-// before is visible to the MMAs that issue() starts, and their results to every thread
-// after.  The group's first warp waits for the others, which only arrive, one of its
-// threads issues, and every warp waits on the mbarrier itself.  (Through two barriers and
-// one waiting thread, the waits at the barriers were the decode's largest stall.)
-// A wait that runs out (1.3 s) marks the thread `dead`: it does not wait again, but keeps
-// the barriers' counts, so that the group comes to its end.
-struct Round {
-  uint64_t* bar;
-  uint32_t parity;
-  int g;
-  bool first, dead;
+// RoundOf's hardware: the named barrier 1 + g of the group's 128 threads, and an mbarrier.
+struct MmaGroup {
+  using Bar = uint64_t*;
+  static __device__ __forceinline__ void before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+  static __device__ __forceinline__ void after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+  static __device__ __forceinline__ void sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
+  static __device__ __forceinline__ void arrive(int g) { asm volatile("bar.arrive %0, 128;" ::"r"(1 + g) : "memory"); }
   template <class Issue>
-  __device__ __forceinline__ void operator()(Issue issue) {
-    start(issue);
-    finish();
-  }
-  template <class Issue>
-  __device__ __forceinline__ void start(Issue issue) {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (first) {
-      asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (elect_one()) {
-        issue();
-        tc::commit(bar);
-      }
-      __syncwarp();
-    } else {
-      asm volatile("bar.arrive %0, 128;" ::"r"(1 + g) : "memory");
+  static __device__ __forceinline__ void issue_and_commit(Issue issue, uint64_t* bar) {
+    if (elect_one()) {
+      issue();
+      tc::commit(bar);
     }
-  }
-  __device__ __forceinline__ void finish() {
-    if (!dead) dead = !tc::wait_bar(bar, parity);
     __syncwarp();
-    parity ^= 1;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  static __device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, tc::wait_bar(bar, parity));
   }
 };
+using Round = RoundOf<MmaGroup>;
 
 __device__ __forceinline__ void fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -433,7 +416,7 @@ __device__ __forceinline__ uint32_t decode_begin(tc::Smem& s, const NeuralDev& n
   // gathers write columns 0..7 only)
   *reinterpret_cast<uint4*>(s.grp[g].a1 + tc::off(row, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
   if (row == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(s.grp[g].bar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.grp[g].bar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (tid < 32) {
@@ -447,11 +430,12 @@ __device__ __forceinline__ uint32_t decode_begin(tc::Smem& s, const NeuralDev& n
   return __shfl_sync(0xffffffffu, s.tmem + 64 * g, 0);
 }
 
-__device__ __forceinline__ void decode_end(tc::Smem& s, const NeuralDev& nd, int warp, bool dead) {
+__device__ __forceinline__ void decode_end(tc::Smem& s, const NeuralDev& nd, int warp, Round& round) {
   cp_async_wait<0>();
+  round.drain();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (dead) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
+  if (round.dead) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "n"(tc::TMEM_COLS));
 }
 
@@ -475,7 +459,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
   const int g = warp >> 2, row = tid & 127;          // group, row of the group's tile
   tc::Group& G = s.grp[g];
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);  // this warp's lanes
-  Round round{G.bar, 0, g, (warp & 3) == 0, false};
+  Round round{&G.bar, 0, g, (warp & 3) == 0, false};
   const uint32_t sb = tc::base_of(&s), a1 = tc::base_of(G.a1), a2 = tc::base_of(G.a2);
   const int64_t ntiles = (a.n + tc::ROWS - 1) / tc::ROWS;
   const int64_t step = 2 * (int64_t)gridDim.x;
@@ -552,7 +536,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     // the next iteration's first group barrier orders these reads of A2 before the
     // next tile writes it
   }
-  decode_end(s, nd, warp, round.dead);
+  decode_end(s, nd, warp, round);
 }
 
 // Deterministic decode on the tensor cores: every tap of the filter window (at one
@@ -632,7 +616,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
   tc::Group& G = s.grp[g];
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
   uint4* arow = reinterpret_cast<uint4*>(G.a1 + tc::off(row, 0, 16));
-  Round round{G.bar, 0, g, (warp & 3) == 0, false};
+  Round round{&G.bar, 0, g, (warp & 3) == 0, false};
   const uint32_t sb = tc::base_of(&s), a1 = tc::base_of(G.a1), a2 = tc::base_of(G.a2);
   constexpr int T2 = Fl::T * Fl::T;
   const int parts = (a.lod != nullptr && nd.nlev > 1 && a.level_mode != STF_LEVEL_NEAREST) ? 2 : 1;
@@ -715,7 +699,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
     }
     cur = nxt;
   }
-  decode_end(s, nd, warp, round.dead);
+  decode_end(s, nd, warp, round);
 }
 
 // ---------------------------------------------------------------- training
@@ -1089,6 +1073,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     for (int o = 16; o > 0; o >>= 1) sums[k] += __shfl_xor_sync(0xffffffffu, sums[k], o);
     if (lane == 0) s.sums[warp][k] = sums[k];
   }
+  round.drain();
   if (row == 0) G.tiles = (int)more;
   if (round.dead) G.abort = 1;
   float* stage = reinterpret_cast<float*>(G.h);       // dW2 64 x 64, then dW3 or dW1 and db 9 x 128
