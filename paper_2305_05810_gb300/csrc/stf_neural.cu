@@ -287,7 +287,7 @@ struct Group {                       // one tile in flight
   unsigned char a1[A1_BYTES];
   unsigned char a2[A2_BYTES];          // H1, then the staged output rows
   uint64_t bar;
-  uint64_t pad;
+  int32_t dead, pad;                   // a warp's wait for an MMA ran out: no more results
 };
 
 struct Smem {
@@ -416,6 +416,7 @@ __device__ __forceinline__ uint32_t decode_begin(tc::Smem& s, const NeuralDev& n
   // gathers write columns 0..7 only)
   *reinterpret_cast<uint4*>(s.grp[g].a1 + tc::off(row, 8, 16)) = make_uint4(0x3C003C00u, 0, 0, 0);
   if (row == 0) {
+    s.grp[g].dead = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.grp[g].bar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -510,14 +511,15 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
 #pragma unroll
     for (int k = 0; k < 7; ++k) v[k] *= cur.sigma;
     const int64_t i = tile * tc::ROWS + row;
-    const bool live = i < a.n;
+    const bool live = i < a.n && !round.dead;
     if (SLIM || a.perm == nullptr) {
       // stage the tile's rows in A2 (free now) and store them coalesced
       float* stage = reinterpret_cast<float*>(G.a2);
 #pragma unroll
       for (int k = 0; k < 7; ++k) stage[row * 7 + k] = v[k];
+      if (round.dead) G.dead = 1;
       group_sync(g);
-      const int nrows = (int)min((int64_t)tc::ROWS, a.n - tile * tc::ROWS);
+      const int nrows = G.dead ? 0 : (int)min((int64_t)tc::ROWS, a.n - tile * tc::ROWS);
       float* dst = a.out + tile * tc::ROWS * 7;
       if (nrows == tc::ROWS && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
         // a full tile: 896 floats as 224 16-byte copies
@@ -693,7 +695,7 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
       if (R >= 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
       if (R >= 32) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
     }
-    if (cur.i < a.n) {
+    if (cur.i < a.n && !round.dead) {
       if (sub < 8 && c < 7) a.out[cur.i * 7 + c] = v[0];
       if (R == 4 && c + 1 < 7) a.out[cur.i * 7 + c + 1] = v[1];
     }
@@ -1038,7 +1040,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
 #pragma unroll
       for (int k = 0; k < 8; ++k) dx[k] = __uint_as_float(q[k]);
     }
-    if (live) {
+    if (live && !round.dead) {
       if (ta.dx_out) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) ta.dx_out[r * 8 + k] = dx[k];
@@ -1132,7 +1134,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       }
     }
   }
-  if (tid < 8) {
+  if (tid < 8 && !aborted) {
     float a = 0.0f;
 #pragma unroll
     for (int w = 0; w < 4 * tct::GROUPS; ++w) a += s.sums[w][tid];
