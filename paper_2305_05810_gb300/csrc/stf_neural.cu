@@ -15,6 +15,7 @@
 #include <math.h>
 
 #include "stf_internal.h"
+#include "stf_memory.h"
 #include "stf_round.h"
 
 namespace stf {
@@ -1381,17 +1382,6 @@ stf_status build_neural(stf_texture_s* t, const stf_neural_desc* d, cudaStream_t
   return STF_OK;
 }
 
-// Whether p lies in memory allocated on a device (not NULL, managed or page-locked host).
-static bool device_memory(const void* p) {
-  cudaPointerAttributes at;
-  if (!p) return false;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeDevice;
-}
-
 static stf_status neural_handle(stf_texture t) {
   if (!handle_ok(t)) return fail(STF_ERR_INVALID_HANDLE, "unknown texture handle");
   if (t->kind != STF_KIND_NEURAL2D) return fail(STF_ERR_UNSUPPORTED, "not a neural texture");
@@ -1415,10 +1405,10 @@ extern "C" stf_status stf_neural_gradients(stf_texture t, const int64_t* ids, in
   ta.target_rows = target_rows;
   ta.batch = batch;
   ta.inv_batch = 1.0f / (float)batch;
-  // straight into the caller's arrays where they are device memory (the atomics do not cross
-  // the host link) and, for the vector atomics, 16-byte aligned
-  const bool direct = (uintptr_t)d_param_grads % 16 == 0 && device_memory(d_param_grads);
-  const bool direct_loss = device_memory(d_loss);
+  // straight into the caller's arrays where they are this device's memory (the atomics cross
+  // neither the host link nor to another device) and, for the vector atomics, 16-byte aligned
+  const bool direct = (uintptr_t)d_param_grads % 16 == 0 && local_memory(d_param_grads);
+  const bool direct_loss = local_memory(d_loss);
   ta.grads = direct ? d_param_grads : t->n_grads;
   ta.loss = direct_loss ? d_loss : t->n_loss;
   ta.dx_out = d_latent_grads;
