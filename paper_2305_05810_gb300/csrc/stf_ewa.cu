@@ -24,6 +24,7 @@ namespace stf {
 
 constexpr int kEwaLut = 128;
 constexpr int kEwaMaxSpan = 4096;   // bounding boxes are far smaller (see ewa_ellipse)
+constexpr float kEwaCondition = 4096.0f;   // largest 4AC/det of ewa_weight2's ellipses
 constexpr int kEwaRows = 48;        // rows whose running sums the stochastic search caches
 
 // Gaussian weight table exp(-2 r) - exp(-2), r = i / 127, rounded to float32.  It is
@@ -79,6 +80,7 @@ struct Ellipse {
   float A, B, C;
   int s0, s1, t0, t1;
   float st_s, st_t;
+  bool plain;             // see ewa_weight2
 };
 
 // Axes at level L in that level's texels; a minor axis longer than 2 texels (only
@@ -105,7 +107,7 @@ __device__ __forceinline__ Ellipse ewa_ellipse(const Footprint& f, float2 uv, fl
   A = __fmul_rn(A, inv);
   B = __fmul_rn(B, inv);
   C = __fmul_rn(C, inv);
-  const float det = __fsub_rn(__fmul_rn(__fmul_rn(4.0f, A), C), __fmul_rn(B, B));
+  const float ac4 = __fmul_rn(__fmul_rn(4.0f, A), C), det = __fsub_rn(ac4, __fmul_rn(B, B));
   const float inv_det = __frcp_rn(det);
   const float hs = __fmul_rn(__fmul_rn(2.0f, inv_det), __fsqrt_rn(__fmul_rn(det, C)));
   const float ht = __fmul_rn(__fmul_rn(2.0f, inv_det), __fsqrt_rn(__fmul_rn(A, det)));
@@ -120,6 +122,8 @@ __device__ __forceinline__ Ellipse ewa_ellipse(const Footprint& f, float2 uv, fl
   e.s1 = (int)floorf(__fadd_rn(e.st_s, hs));
   e.t0 = (int)ceilf(__fsub_rn(e.st_t, ht));
   e.t1 = (int)floorf(__fadd_rn(e.st_t, ht));
+  e.plain = det > 0.0f && ac4 <= __fmul_rn(kEwaCondition, det) && ac4 < 3.4e38f && fabsf(e.st_s) < 8380000.0f &&
+            fabsf(e.st_t) < 8380000.0f;
   return e;
 }
 
@@ -151,10 +155,16 @@ __device__ __forceinline__ float ewa_weight(const Ellipse& e, const float* lut, 
 }
 
 // The weights of texels is and is + 1 (x = their float coordinates) of a row: the same
-// operations and roundings as ewa_weight, for an ellipse with ewa_plain().  The second
-// texel may lie past the box's end, where its weight is 0 without a test: the box ends
-// where Q reaches 1, to a relative error far below 1/128, and the table's last entry
-// (Q from 127/128) is exactly 0.  Float counters
+// operations and roundings as ewa_weight, for an ellipse that is `plain`: coordinates that
+// count up exactly in float32, and k = 4AC/det at most 4096.  The second texel may lie past
+// the box's end, and its weight must be 0 there without a test: the table's last entry, of Q
+// from 127/128, is exactly 0.  det's float32 cancellation makes the box's half width short by
+// at most k 2^-24, and Q's own roundings lower it by at most 15 k 2^-24, so Q past the box
+// is at least 1 - 17 k 2^-24: above 127/128 for k up to 7700.  Footprints of a major and a
+// minor axis have k below 820 (axes' ratio 64, minor axis 2 texels); a long one without any
+// minor axis, or at the 1-texel levels of a long texture, has more and takes the checked
+// loops, as do coefficients that are not finite and det = 0, whose box is not theirs.
+// Float counters
 // replace the integer conversions, the last addition saturates (Q < 0 counts as 0; Q >= 1
 // becomes 1, whose entry lut[128] is 0), and adding 2^23 rounding towards zero leaves the
 // table index in the low mantissa bits.  9 issued instructions a texel, against 14 with
@@ -188,13 +198,6 @@ __device__ __forceinline__ float2 ewa_weight2(const Ellipse& e, uint32_t lut, fl
 // Shared-memory address of the table, less the offset that 2^23's bits add (modulo 2^32).
 __device__ __forceinline__ uint32_t ewa_lut_base(const float* lut) {
   return (uint32_t)__cvta_generic_to_shared(lut) - (0x4B000000u << 2);
-}
-
-// Finite coefficients, and coordinates that count up exactly in float32.  Other ellipses
-// (derivatives near the float32 range, uv beyond 2^23 texels) take the checked loops.
-__device__ __forceinline__ bool ewa_plain(const Ellipse& e) {
-  return fabsf(e.st_s) < 8380000.0f && fabsf(e.st_t) < 8380000.0f && fabsf(e.A) <= 3.4e38f && fabsf(e.B) <= 3.4e38f &&
-         fabsf(e.C) <= 3.4e38f;
 }
 
 struct EwaLevel {
@@ -375,7 +378,7 @@ __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable ta
           int cs = 0, ct = 0;
           const float u = unit24(r.x);
           bool found;
-          if (ewa_plain(e)) {
+          if (e.plain) {
             found = ewa_choose<true>(e, lut, u, cs, ct);
           } else {
             int s2 = 0, t2 = 0;
@@ -411,7 +414,7 @@ __global__ void __launch_bounds__(256) k_ewa(Tex2DView t, EwaArgs a, EwaTable ta
             continue;
           }
           float acc[C], S;
-          if (ewa_plain(e)) {
+          if (e.plain) {
             S = ewa_average<FMT, C, true>(t, L, lv, e, lut, acc);
           } else {
             float a2[C];

@@ -231,3 +231,51 @@ def test_ewa_far_coordinates_match_oracle(scale):
     ok = np.isfinite(tol)
     assert np.all(np.abs(det - dv)[ok] <= (2e-6 * np.abs(dv) + tol[:, None])[ok])
     stf.stf_synchronize(T.handle)
+
+
+def _box32(uv, g, size):
+    """Level-0 coefficients, position and box of float32 footprints without a minor axis, in
+    the documented order of float32 operations."""
+    f = np.float32
+    u, v = g[:, 0] * f(size), g[:, 1] * f(size)
+    A, B, C = v * v + f(0) + f(1), f(-2) * (u * v + f(0)), u * u + f(0) + f(1)
+    inv = f(1) / (A * C - (B * B) * f(0.25))
+    A, B, C = A * inv, B * inv, C * inv
+    det = f(4) * A * C - B * B
+    inv = f(1) / det
+    hs, ht = f(2) * inv * np.sqrt(det * C), f(2) * inv * np.sqrt(A * det)
+    s, t = uv[:, 0] * f(size) - f(0.5), uv[:, 1] * f(size) - f(0.5)
+    return A, B, C, s, t, np.floor(s + hs), np.ceil(t - ht), np.floor(t + ht)
+
+
+def test_ewa_texels_past_the_box_have_no_weight():
+    """Footprints with one zero derivative, 1000 to 2040 texels long: det cancels, the box comes
+    out short, and the texel past its end lies inside the ellipse.  The steps end at the box:
+    in a texture that is zero but for that texel's column, the average is exactly zero.  The
+    last footprint's 4AC - B^2 overflows: its box is texel (0, 0) alone."""
+    size, m = 4096, 3000
+    rng = np.random.default_rng(6)
+    uv = rng.uniform(0.1, 0.6, (m, 2)).astype(np.float32)
+    g = np.zeros((m, 4), np.float32)
+    ang, length = rng.uniform(0, 2 * np.pi, m), rng.uniform(1000, 2040, m)
+    g[:, 0], g[:, 1] = np.cos(ang) * length / size, np.sin(ang) * length / size
+    uv[0], g[0] = (0.6688878, 0.23138922), (0.2908255287, 0.2427806917, 0, 0)
+    A, B, C, s, t, s1, t0, t1 = _box32(uv, g, size)
+    past = []
+    for i in range(m):
+        tt = np.arange(t0[i], t1[i] + 1).astype(np.float32) - t[i]
+        ss = np.float32(s1[i] + 1) - s[i]
+        if ((A[i] * ss + B[i] * tt) * ss + C[i] * (tt * tt)).min() < 127 / 128 and 1 < s1[i] < size - 3:
+            past.append(i)
+    assert 0 in past and len(past) >= 5
+    texels = torch.zeros((size, size, 1), device=dev())
+    cases = [(uv[i], g[i], int(s1[i]) + 1) for i in past[:8]]
+    cases.append((np.float32([0.5, 0.5]), np.float32([1.79e19 / size, 0.45 / size, 0, 0]), 1))
+    for p, d, column in cases:
+        texels.zero_()
+        texels[:, column] = 1.0
+        T = stf.Texture(stf.KIND_TEX2D, texels, dims=(size, size, 1), channels=1)
+        got = T.lookup_ewa_deterministic(to_dev(p[None]), to_dev(d[None]), 16.0)
+        stf.stf_synchronize(T.handle)
+        assert float(got) == 0.0, (p, d, column, float(got))
+        T.close()
