@@ -70,7 +70,6 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 struct NeuralPick {
   int64_t j;      // caller's query slot
   float sigma;    // estimator scale (Catmull-Rom)
-  int4 tap;
   int mode;       // 0: no texel (background), 1: decode the latent, 2: stored fallback texel
 };
 
@@ -99,7 +98,6 @@ __device__ __forceinline__ NeuralPick neural_pick(const NeuralDev& nd, const Loo
   NeuralPick pk;
   pk.j = 0;
   pk.sigma = 1.0f;
-  pk.tap = make_int4(0, 0, 0, -1);
   pk.mode = 0;
   if (i >= a.n) return pk;
   pk.j = SLIM ? i : query_slot(a, i);
@@ -114,10 +112,12 @@ __device__ __forceinline__ NeuralPick neural_pick(const NeuralDev& nd, const Loo
   }
   const int w = nd.lvl_w[L], h = nd.lvl_h[L];
   float x[2] = {__fsub_rn(__fmul_rn(uv.x, (float)w), 0.5f), __fsub_rn(__fmul_rn(uv.y, (float)h), 0.5f)};
-  if (!(prepare_coords<2>(x) && isfinite(lod))) return pk;
-  int idx[2];
-  pk.sigma = pick_taps_r<F, 2, false>(x, r, idx);
-  pk.tap = make_int4(idx[0], idx[1], 0, L);
+  const bool ok = prepare_coords<2>(x) && isfinite(lod);
+  int idx[2] = {0, 0};
+  if (ok) pk.sigma = pick_taps_r<F, 2, false>(x, r, idx);
+  // (the tap goes out here: carried to the tile's end, two tiles' taps were eight registers)
+  if (!SLIM && a.taps) reinterpret_cast<int4*>(a.taps)[pk.j] = ok ? make_int4(idx[0], idx[1], 0, L) : make_int4(0, 0, 0, -1);
+  if (!ok) return pk;
   const int cx = min(max(idx[0], 0), w - 1), cy = min(max(idx[1], 0), h - 1);
   const __half* base = L < nd.nlat ? nd.lat16 : nd.fb16;
   cp_async16(row, base + (nd.lvl_off[L] + (int64_t)cy * w + cx) * 8);
@@ -288,7 +288,7 @@ struct Group {                       // one tile in flight
   unsigned char a1[A1_BYTES];
   unsigned char a2[A2_BYTES];          // H1, then the staged output rows
   uint64_t bar;
-  int32_t dead, pad;                   // a warp's wait for an MMA ran out: no more results
+  int32_t dead, pad;                   // a warp gave up: its rows of the staged ones are not there
 };
 
 struct Smem {
@@ -432,9 +432,8 @@ __device__ __forceinline__ uint32_t decode_begin(tc::Smem& s, const NeuralDev& n
   return __shfl_sync(0xffffffffu, s.tmem + 64 * g, 0);
 }
 
-__device__ __forceinline__ void decode_end(tc::Smem& s, const NeuralDev& nd, int warp, Round& round) {
+__device__ __forceinline__ void decode_end(tc::Smem& s, const NeuralDev& nd, int warp, const Round& round) {
   cp_async_wait<0>();
-  round.drain();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (round.dead) atomicOr(nd.status, STF_DEV_MMA_TIMEOUT);
@@ -472,12 +471,16 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
   cp_async_commit();
   // coordinates of the next tile, loaded a whole tile ahead of its tap choice
   QueryCoords qn = load_coords(a, (tile + step) * tc::ROWS + row);
+  // barrier phases of a tile, and those still to come in it where a wait runs out
+  const int phases = SLIM || a.perm == nullptr ? 4 : 3;
+  int left = -1;
   for (; tile < ntiles; tile += step) {
     cp_async_wait<0>();
     uint4 fb = make_uint4(0, 0, 0, 0);
     if (cur.mode == 2) fb = *arow;                   // stored fallback texel (own row)
     fence_smem();
-    round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); });
+    left = phases - 1;
+    if (!round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); })) break;
     tc_hidden(trow, G.a2, row);
     fence_smem();
     round.start([&] { tc_layer2<tc::Smem>(tmem, sb, a2, 64); });
@@ -487,9 +490,12 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     if (next < ntiles) nxt = neural_pick<F, SLIM>(nd, a, next * tc::ROWS + row, arow, &qn);
     cp_async_commit();
     qn = load_coords(a, (next + step) * tc::ROWS + row);
-    round.finish();
+    left = phases - 2;
+    if (!round.finish()) break;
     tc_hidden_tmem(trow);
-    round([&] { tc_layer3<tc::Smem>(tmem, sb); });
+    left = phases - 3;
+    if (!round([&] { tc_layer3<tc::Smem>(tmem, sb); })) break;
+    left = -1;
     float v[8];
     {
       uint32_t r[8];
@@ -511,14 +517,11 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
     }
 #pragma unroll
     for (int k = 0; k < 7; ++k) v[k] *= cur.sigma;
-    const int64_t i = tile * tc::ROWS + row;
-    const bool live = i < a.n && !round.dead;
     if (SLIM || a.perm == nullptr) {
       // stage the tile's rows in A2 (free now) and store them coalesced
       float* stage = reinterpret_cast<float*>(G.a2);
 #pragma unroll
       for (int k = 0; k < 7; ++k) stage[row * 7 + k] = v[k];
-      if (round.dead) G.dead = 1;
       group_sync(g);
       const int nrows = G.dead ? 0 : (int)min((int64_t)tc::ROWS, a.n - tile * tc::ROWS);
       float* dst = a.out + tile * tc::ROWS * 7;
@@ -530,14 +533,17 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
       } else {
         for (int e = row; e < nrows * 7; e += 128) dst[e] = stage[e];
       }
-    } else if (live) {
+    } else if (tile * tc::ROWS + row < a.n) {
 #pragma unroll
       for (int k = 0; k < 7; ++k) a.out[cur.j * 7 + k] = v[k];
     }
-    if (!SLIM && live && a.taps) reinterpret_cast<int4*>(a.taps)[cur.j] = cur.tap;
     cur = nxt;
     // the next iteration's first group barrier orders these reads of A2 before the
     // next tile writes it
+  }
+  if (left >= 0) {
+    G.dead = 1;
+    round.give_up(left, phases, tile, ntiles, step);
   }
   decode_end(s, nd, warp, round);
 }
@@ -550,10 +556,9 @@ __global__ void __launch_bounds__(256, 4) k_neural_stochastic_tc(NeuralDev nd, L
 // three layers run as in the stochastic decode, and each row's output times its
 // weight (the tap weights wx wy times the level weight) is summed over the query's R
 // rows.  Fallback levels use the stored texel.
-// One row of a deterministic tile: its query, weight and texel kind.  The texel (latent
+// One row of a deterministic tile: its weight and texel kind.  The texel (latent
 // or stored fallback) is gathered into the row of the A tile by cp.async.
 struct DetRow {
-  int64_t i;     // query
   float w;       // tap weight times level weight (0: the row adds nothing)
   int mode;      // 0: nothing, 1: decode the latent, 2: stored fallback texel
 };
@@ -563,7 +568,6 @@ __device__ __forceinline__ DetRow det_row(const NeuralDev& nd, const LookupArgs&
                                           int ty, uint4* arow, const QueryCoords* pre = nullptr) {
   using Fl = Filter<F>;
   DetRow d;
-  d.i = i;
   d.w = 0.0f;
   d.mode = 0;
   if (i >= a.n) return d;
@@ -634,13 +638,15 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
   if (tile < ntiles) cur = det_row<F>(nd, a, tile * Q + qi, p, tx, ty, arow);
   cp_async_commit();
   QueryCoords qn = load_coords(a, (tile + step) * Q + qi);        // a tile ahead
+  int left = -1;                               // barrier phases still to come in the tile, where a wait runs out
   for (; tile < ntiles; tile += step) {
     cp_async_wait<0>();
     uint4 fb = make_uint4(0, 0, 0, 0);
     if (cur.mode == 2) fb = *arow;               // stored fallback texel (own row)
     if (cur.mode != 1) *arow = make_uint4(0, 0, 0, 0);
     fence_smem();
-    round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); });
+    left = 2;
+    if (!round([&] { tc_layer1<tc::Smem>(tmem, sb, a1); })) break;
     tc_hidden(trow, G.a2, row);
     fence_smem();
     round.start([&] { tc_layer2<tc::Smem>(tmem, sb, a2, 64); });
@@ -650,9 +656,12 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
     if (next < ntiles) nxt = det_row<F>(nd, a, next * Q + qi, p, tx, ty, arow, &qn);
     cp_async_commit();
     qn = load_coords(a, (next + step) * Q + qi);
-    round.finish();
+    left = 1;
+    if (!round.finish()) break;
     tc_hidden_tmem(trow);
-    round([&] { tc_layer3<tc::Smem>(tmem, sb); });
+    left = 0;
+    if (!round([&] { tc_layer3<tc::Smem>(tmem, sb); })) break;
+    left = -1;
     float v[8];
     {
       uint32_t r[8];
@@ -696,12 +705,14 @@ __global__ void __launch_bounds__(256, 4) k_neural_deterministic_tc(NeuralDev nd
       if (R >= 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
       if (R >= 32) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
     }
-    if (cur.i < a.n && !round.dead) {
-      if (sub < 8 && c < 7) a.out[cur.i * 7 + c] = v[0];
-      if (R == 4 && c + 1 < 7) a.out[cur.i * 7 + c + 1] = v[1];
+    const int64_t i = tile * Q + qi;
+    if (i < a.n) {
+      if (sub < 8 && c < 7) a.out[i * 7 + c] = v[0];
+      if (R == 4 && c + 1 < 7) a.out[i * 7 + c + 1] = v[1];
     }
     cur = nxt;
   }
+  if (left >= 0) round.give_up(left, 3, tile, ntiles, step);
   decode_end(s, nd, warp, round);
 }
 
@@ -957,6 +968,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
   using S = tct::Smem;
   float sums[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // db3, sum of squared errors
   uint32_t more = 0;                          // 0 for the group's first tile: accumulators start from zero
+  int left = -1;                              // barrier phases still to come in the tile, where a wait runs out
   for (; tile < ntiles; tile += step) {
     const int64_t r = tile * 128 + row;
     const bool live = cur.live;
@@ -964,20 +976,23 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     *reinterpret_cast<uint4*>(G.x + tc::off(row, 0, 16)) =
         make_uint4(pack_h2(X[0], X[1]), pack_h2(X[2], X[3]), pack_h2(X[4], X[5]), pack_h2(X[6], X[7]));
     fence_smem();
-    round([&] { tc_layer1<S>(tmem, sb, gx); });
+    left = 5;
+    if (!round([&] { tc_layer1<S>(tmem, sb, gx); })) break;
     tct_hidden(trow, G.h, 0, row);
     fence_smem();
-    round([&] { tc_layer2<S>(tmem, sb, gh, 128); });
+    left = 4;
+    if (!round([&] { tc_layer2<S>(tmem, sb, gh, 128); })) break;
     tct_hidden(trow, G.h, 64, row);
     fence_smem();
-    round([&] {
+    left = 3;
+    if (!round([&] {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         tc::mma(tmem, tc::desc_at(gh, 1024 + kk * 256, 128), tc::desc_at(sb, offsetof(S, b3) + kk * 256, 64),
                 tc::idesc(128, 16), kk);
       tc::mma(tmem, tc::desc_rows_repeated(sb, offsetof(S, ones)), tc::desc_at(sb, offsetof(S, b3x), 16),
               tc::idesc(128, 16), 1);
-    });
+    })) break;
     {
       uint32_t y[8];
       tc::tmem_ld<8>(trow, y);
@@ -1002,16 +1017,18 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     TrainRow nxt;
     nxt.load(nd, ta, (tile + step) * 128 + row);
     fence_smem();
-    round([&] {
+    left = 2;
+    if (!round([&] {
       tc::mma(tmem, tc::desc_at(gdy, 0, 16), tc::desc_at(sb, offsetof(S, r3), 16), tc::idesc(128, 64), 0);
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         tc::mma(tmem + tct::C_W3, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gdy, 0, j, 16), tct::idesc_mn(128, 16),
                 more | j);
-    });
+    })) break;
     tct_masked(trow, G.h, 64, row);
     fence_smem();
-    round([&] {
+    left = 1;
+    if (!round([&] {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         tc::mma(tmem, tc::desc_at(gh, 1024 + kk * 256, 128), tc::desc_at(sb, offsetof(S, r2) + kk * 256, 64),
@@ -1020,10 +1037,11 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       for (int j = 0; j < 8; ++j)
         tc::mma(tmem + tct::C_W2, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gh, 64, j, 128), tct::idesc_mn(128, 64),
                 more | j);
-    });
+    })) break;
     tct_masked(trow, G.h, 0, row);
     fence_smem();
-    round([&] {
+    left = 0;
+    if (!round([&] {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         tc::mma(tmem, tc::desc_at(gh, kk * 256, 128), tc::desc_at(sb, offsetof(S, r1) + kk * 256, 64),
@@ -1032,7 +1050,8 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
       for (int j = 0; j < 8; ++j)
         tc::mma(tmem + tct::C_W1, tct::desc_mn(gh, 0, j, 128), tct::desc_mn(gx, 0, j, 16), tct::idesc_mn(128, 16),
                 more | j);
-    });
+    })) break;
+    left = -1;
     more = 1;
     float dx[8];
     {
@@ -1041,7 +1060,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
 #pragma unroll
       for (int k = 0; k < 8; ++k) dx[k] = __uint_as_float(q[k]);
     }
-    if (live && !round.dead) {
+    if (live) {
       if (ta.dx_out) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) ta.dx_out[r * 8 + k] = dx[k];
@@ -1068,6 +1087,7 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     }
     cur = nxt;
   }
+  if (left >= 0) round.give_up(left, 6, tile, ntiles, step);
   // The groups' gradients: groups 1 and 2 leave their rows in their own tiles, [column]
   // [row], group 0 adds them to its own and takes them to memory.
 #pragma unroll
@@ -1076,7 +1096,6 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
     for (int o = 16; o > 0; o >>= 1) sums[k] += __shfl_xor_sync(0xffffffffu, sums[k], o);
     if (lane == 0) s.sums[warp][k] = sums[k];
   }
-  round.drain();
   if (row == 0) G.tiles = (int)more;
   if (round.dead) G.abort = 1;
   float* stage = reinterpret_cast<float*>(G.h);       // dW2 64 x 64, then dW3 or dW1 and db 9 x 128

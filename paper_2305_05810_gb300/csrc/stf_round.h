@@ -17,25 +17,25 @@ namespace stf {
 // every warp waits on the mbarrier itself.  (Through two barriers and one waiting thread,
 // the waits at the barriers were the decode's largest stall.)
 //
-// A warp whose wait runs out is `dead`: it waits for no MMA and issues none any more, but
-// goes on to the end of its tiles and takes the barrier of every round, so that the group's
-// other warps come to theirs.  At the barriers a dead warp waits for the phase to end: if it
-// only arrived, it would come by again before the first warp has been there once, and the
-// phases it ended in the first warp's place would leave that warp waiting for good.  (A warp
-// that is not dead cannot come by twice: it waits for the MMAs that the first warp issues
-// after the phase's end, with a limit far beyond what the first warp does in between.)
-// Results of a dead warp are not to be stored.
+// finish() is false, in all lanes, when the warp's wait ran out.  The warp then leaves its
+// tiles, issues, reads and stores nothing more, and takes the barrier phases that it has left
+// with give_up(), so that the group's other warps come to the end of theirs.  There it waits
+// for each phase to end: if it only arrived, it would come by again before the first warp has
+// been there once, and the phases that ended in the first warp's place would leave that warp
+// waiting for good.  (A warp that goes on cannot come by twice: it waits for the MMAs that the
+// first warp issues after the phase's end, with a limit far beyond what the first warp does in
+// between.)  A flag that every round tests instead made the decodes 2 to 3% slower.
 template <class Hw>
 struct RoundOf {
   typename Hw::Bar bar;
-  uint32_t parity;             // of the MMAs to wait for, also by drain() when dead
+  uint32_t parity;
   int g;                       // group
   bool first, dead;            // (the same in all lanes)
 
   template <class Issue>
-  STF_ROUND_FN void operator()(Issue issue) {
+  STF_ROUND_FN bool operator()(Issue issue) {
     start(issue);
-    finish();
+    return finish();
   }
 
   template <class Issue>
@@ -44,25 +44,32 @@ struct RoundOf {
     if (first) {
       Hw::sync(g);
       Hw::after_sync();
-      if (!dead) Hw::issue_and_commit(issue, bar);
-    } else if (dead) {
-      Hw::sync(g);
+      Hw::issue_and_commit(issue, bar);
     } else {
       Hw::arrive(g);
     }
   }
 
-  STF_ROUND_FN void finish() {
-    if (!dead) {
-      dead = !Hw::wait(bar, parity);
-      if (!dead) parity ^= 1;
-    }
+  STF_ROUND_FN bool finish() {
+    const bool done = Hw::wait(bar, parity);
+    parity ^= 1;
     Hw::after_sync();
+    return done;
   }
 
-  // Before the group gives up its tiles: once more the wait that ran out.
-  STF_ROUND_FN void drain() {
-    if (dead) Hw::wait(bar, parity);
+  // After a finish() that was false: takes the `left` barrier phases still to come in the tile
+  // and `phases` for each tile after it, and waits once more for the MMAs before the group
+  // gives up its tiles.
+  template <class I>
+  STF_ROUND_FN void give_up(int left, int phases, I tile, I tiles, I step) {
+    dead = true;
+    for (;;) {
+      for (; left > 0; --left) Hw::sync(g);
+      tile += step;
+      if (tile >= tiles) break;
+      left = phases;
+    }
+    Hw::wait(bar, parity ^ 1);
   }
 };
 

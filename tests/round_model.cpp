@@ -26,7 +26,7 @@ struct Model {
 };
 
 static Model* model;
-thread_local int warp, round_no, gave_up_at, issued_dead;
+thread_local int warp, round_no, gave_up_at;
 
 static void fail(const char* what) {
   std::printf("%s: warp %d, round %d; late", what, warp, round_no);
@@ -72,44 +72,46 @@ struct HostGroup {
   // of round round_no (of the one that was given up, when it is waited for again)
   static bool wait(int, uint32_t parity) {
     std::unique_lock<std::mutex> lk(model->m);
-    const int r = gave_up_at >= 0 ? gave_up_at : round_no;
+    const bool again = gave_up_at >= 0;
+    const int r = again ? gave_up_at : round_no;
     if (parity != (uint32_t)(r & 1)) fail("waits for another phase");
-    if (gave_up_at < 0) until(lk, "the first warp never comes", [](int n) { return model->phases > n; }, r);
-    if (model->lost(r) || (gave_up_at < 0 && model->late[warp] == r)) {
-      gave_up_at = r;
-      return false;
-    }
+    if (!again) until(lk, "the first warp never comes", [](int n) { return model->phases > n; }, r);
     // complete once issued; the first warp issues right after the phase's end or not at all
-    if (!model->cv.wait_for(lk, std::chrono::milliseconds(20), [&] { return model->issued > r; })) {
-      gave_up_at = r;
-      return false;
-    }
-    return true;
+    const bool done = !model->lost(r) && !(!again && model->late[warp] == r) &&
+                      model->cv.wait_for(lk, std::chrono::milliseconds(20), [&] { return model->issued > r; });
+    if (!done) gave_up_at = r;
+    return done;
   }
 };
 
-static void warp_main(int w, int rounds) {
+// Tiles of PHASES rounds each, as the kernels walk them.
+constexpr int PHASES = 3;
+
+static void warp_main(int w, int tiles) {
   warp = w;
   gave_up_at = -1;
+  round_no = 0;
   stf::RoundOf<HostGroup> round{0, 0, 0, w == 0, false};
-  for (round_no = 0; round_no < rounds; ++round_no) {
-    const bool was_dead = round.dead;
-    round([&] { if (was_dead) fail("a dead warp issues"); });
-    if (was_dead && !round.dead) fail("a dead warp comes back");
-    if (gave_up_at >= 0 && !round.dead) fail("a wait ran out and the warp goes on");
-  }
-  round.drain();
+  int tile = 0, left = -1;
+  for (; tile < tiles && left < 0; left < 0 ? ++tile : 0)
+    for (int k = 0; k < PHASES; ++k, ++round_no)
+      if (!round([] {})) {
+        left = PHASES - 1 - k;
+        break;
+      }
+  if (left >= 0) round.give_up(left, PHASES, tile, tiles, 1);
+  if (round.dead != (gave_up_at >= 0)) fail("a wait ran out and the warp goes on");
 }
 
 int main(int argc, char** argv) {
-  const int rounds = argc > 1 ? std::atoi(argv[1]) : 5;
+  const int tiles = argc > 1 ? std::atoi(argv[1]) : 2, rounds = PHASES * tiles;
   auto run = [&](const int* late, int lost) {
     Model mm;
     for (int w = 0; w < WARPS; ++w) mm.late[w] = late[w];
     mm.lost_round = lost;
     model = &mm;
     std::vector<std::thread> t;
-    for (int w = 0; w < WARPS; ++w) t.emplace_back(warp_main, w, rounds);
+    for (int w = 0; w < WARPS; ++w) t.emplace_back(warp_main, w, tiles);
     for (auto& x : t) x.join();
     if (mm.arrived != 0 || mm.phases != rounds) fail("arrivals left over");
   };

@@ -20,7 +20,7 @@ def model(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("rounds", [1, 2, 3, 7])
-def test_every_warp_comes_to_its_end(model, rounds):
-    r = subprocess.run([model, str(rounds)], capture_output=True, text=True, timeout=300)
+@pytest.mark.parametrize("tiles", [1, 2, 3])
+def test_every_warp_comes_to_its_end(model, tiles):
+    r = subprocess.run([model, str(tiles)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout
