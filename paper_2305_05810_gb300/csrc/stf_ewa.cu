@@ -172,7 +172,7 @@ __device__ __forceinline__ float ewa_weight(const Ellipse& e, const float* lut, 
 // forms (5.4 M queries of a 4K ground plane: 130 -> 107 us stochastic, 153 -> 133 us
 // deterministic).
 __device__ __forceinline__ float ewa_lut_at(uint32_t lut, float r2x128) {
-  // (no volatile: the table does not change after it was staged)
+  // (no volatile: the table does not change after it was staged, which ewa_lut_base waits for)
   float w;
   asm("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(lut + (__float_as_uint(r2x128) << 2)));
   return w;
@@ -196,8 +196,12 @@ __device__ __forceinline__ float2 ewa_weight2(const Ellipse& e, uint32_t lut, fl
 }
 
 // Shared-memory address of the table, less the offset that 2^23's bits add (modulo 2^32).
+// The volatile statement keeps its place after the barrier that ends the staging, and
+// ewa_lut_at's reads, which nothing else ties to that barrier, depend on it.
 __device__ __forceinline__ uint32_t ewa_lut_base(const float* lut) {
-  return (uint32_t)__cvta_generic_to_shared(lut) - (0x4B000000u << 2);
+  uint32_t base = (uint32_t)__cvta_generic_to_shared(lut) - (0x4B000000u << 2);
+  asm volatile("" : "+r"(base)::"memory");
+  return base;
 }
 
 struct EwaLevel {
