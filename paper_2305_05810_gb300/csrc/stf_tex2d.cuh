@@ -194,14 +194,6 @@ __device__ __forceinline__ DetLevels det_levels(const Tex2DView& t, const Lookup
   return d;
 }
 
-// The same at uv.
-template <int F, int FMT, int C>
-__device__ __forceinline__ void tex2d_det_uv(const Tex2DView& t, int L, float2 uv, float scale, float width, float* acc) {
-  float x[2] = {__fsub_rn(__fmul_rn(uv.x, (float)t.level_w[L]), 0.5f),
-                __fsub_rn(__fmul_rn(uv.y, (float)t.level_h[L]), 0.5f)};
-  if (prepare_coords<2>(x)) tex2d_det_level<F, FMT, C>(t, L, x, scale, width, acc);
-}
-
 // ---------------------------------------------------------------- triplanar
 
 struct Planes {
@@ -461,45 +453,43 @@ __global__ void __launch_bounds__(256) k_tex2d_stochastic(Tex2DView t, LookupArg
 // whose queries lie apart each read 32 lines, and the L1 data pipe bounds the filter (96%
 // busy).  Such a warp runs its queries in four rounds of eight instead, four lanes to a
 // query, one per tap column: the lanes read the four neighbouring texels of a row in one
-// load, and their partial sums meet by halving exchanges.  A warp whose queries are
-// neighbours shares lines between lanes already and keeps one thread per query, which
-// sets up its weights once instead of four times.  4.2 M random lookups of a 256^2 FP32
-// RGBA texture: 168 -> 103 us; in raster order unchanged (54 us; 94 us by columns).
+// load, and their partial sums meet by halving exchanges.  Queries that are neighbours share
+// lines between lanes already and keep one thread each, which sets up its weights once
+// instead of four times.  4.2 M lookups of a 256^2 FP32 RGBA texture: 168 -> 104 us at random
+// points, 58 -> 52 us in raster order (94 us by columns); half random and then in raster order
+// 111 -> 77 us (101 us when a warp's first queries decided for all of its later ones).
 
-// Raster position of a query at level L, and whether it takes part.
-struct RasterPos {
-  float x[2];
-  int L;
-  bool on;
-  __device__ __forceinline__ RasterPos(const Tex2DView& t, int L_, float2 uv, bool ok) : L(L_) {
-    x[0] = __fsub_rn(__fmul_rn(uv.x, (float)t.level_w[L]), 0.5f);
-    x[1] = __fsub_rn(__fmul_rn(uv.y, (float)t.level_h[L]), 0.5f);
-    on = ok && prepare_coords<2>(x);
+// The window at raster position (x, y) of level L with its weights times `scale`.
+template <int F, int FMT, int C>
+struct CubicWindow {
+  int L, W, H, bx, by;
+  float wx[4], wy[4];
+  __device__ __forceinline__ CubicWindow(const Tex2DView& t, int L_, float x, float y, float scale) : L(L_) {
+    using Fl = Filter<F>;
+    W = t.level_w[L];
+    H = t.level_h[L];
+    float fx, fy;
+    bx = axis_base(x, fx) + Fl::OFF0;
+    by = axis_base(y, fy) + Fl::OFF0;
+    Fl::weights(fx, wx);
+    Fl::weights(fy, wy);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) wy[k] *= scale;
+  }
+  // Column k, added to acc.
+  __device__ __forceinline__ void column(const Tex2DView& t, int k, float* acc) const {
+    const float wk = k == 0 ? wx[0] : k == 1 ? wx[1] : k == 2 ? wx[2] : wx[3];
+    const int cx = min(max(bx + k, 0), W - 1);
+#pragma unroll
+    for (int ky = 0; ky < 4; ++ky) {
+      float tv[C];
+      fetch2d<FMT, C>(t, L, cx, min(max(by + ky, 0), H - 1), tv);
+      const float w = wk * wy[ky];
+#pragma unroll
+      for (int c = 0; c < C; ++c) acc[c] = fmaf(w, tv[c], acc[c]);
+    }
   }
 };
-
-// Column k of the window at raster position (x, y) of level L, weighted by `scale`, added
-// to acc.
-template <int F, int FMT, int C>
-__device__ __forceinline__ void tex2d_det_column(const Tex2DView& t, int L, float x, float y, float scale, int k,
-                                                 float* acc) {
-  using Fl = Filter<F>;
-  const int W = t.level_w[L], H = t.level_h[L];
-  float fx, fy, wx[4], wy[4];
-  const int bx = axis_base(x, fx) + Fl::OFF0, by = axis_base(y, fy) + Fl::OFF0;
-  Fl::weights(fx, wx);
-  Fl::weights(fy, wy);
-  const float wk = k == 0 ? wx[0] : k == 1 ? wx[1] : k == 2 ? wx[2] : wx[3];
-  const int cx = min(max(bx + k, 0), W - 1);
-#pragma unroll
-  for (int ky = 0; ky < 4; ++ky) {
-    float tv[C];
-    fetch2d<FMT, C>(t, L, cx, min(max(by + ky, 0), H - 1), tv);
-    const float w = wk * (wy[ky] * scale);
-#pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = fmaf(w, tv[c], acc[c]);
-  }
-}
 
 // One thread per query: the loop of the filters that do not gather by warp.
 template <int F, int FMT, int C, typename I>
@@ -516,58 +506,88 @@ __device__ __forceinline__ void tex2d_det_loop(const Tex2DView& t, const LookupA
   }
 }
 
-// At most kFastLoopMaxQueries queries; a warp's first ones decide how it takes all of its
-// queries.  With levels of detail
-// only texels of 16 bytes and more gain (8-channel FP16 122 us against 136, 4-channel FP16
-// 105 against 90 for 2.1 M queries at random levels: the second level's setup is paid
-// four times as well).
-template <int F, int FMT, int C>
-__global__ void __launch_bounds__(256) k_tex2d_cubic(Tex2DView t, LookupArgs a) {
+// A query's window positions: at level 0, or (LEVELS) at one or two levels with their
+// weights.  A part that adds nothing has level -1.
+template <bool LEVELS>
+struct CubicParts {
+  static constexpr int N = LEVELS ? 2 : 1;
+  int L[N];
+  float x[N], y[N], w[N];
+  __device__ __forceinline__ CubicParts(const Tex2DView& t, const LookupArgs& a, float2 uv, float lod, bool live) {
+    L[0] = live && isfinite(lod) ? 0 : -1;
+    w[0] = 1.0f;
+    if constexpr (LEVELS) {
+      const DetLevels d = det_levels(t, a, lod);
+      L[0] = live && d.w0 > 0.0f ? d.L0 : -1;
+      L[1] = live && d.w1 > 0.0f ? d.L1 : -1;
+      w[0] = d.w0;
+      w[1] = d.w1;
+    }
+#pragma unroll
+    for (int p = 0; p < N; ++p) {
+      const int l = LEVELS ? max(L[p], 0) : 0;
+      float q[2] = {__fsub_rn(__fmul_rn(uv.x, (float)t.level_w[l]), 0.5f),
+                    __fsub_rn(__fmul_rn(uv.y, (float)t.level_h[l]), 0.5f)};
+      if (!prepare_coords<2>(q)) L[p] = -1;
+      x[p] = q[0];
+      y[p] = q[1];
+    }
+  }
+};
+
+// At most kFastLoopMaxQueries queries.  Both ways of a warp's 32 queries sum a column's texels
+// in the same order (of both levels), then columns 0 and 2, 1 and 3, and the two sums: a
+// query's value does not depend on the queries beside it.
+// (Four FP16 channels on six blocks an SM, 40 registers: raster order 56 -> 54 us.)
+template <int F, int FMT, int C, bool LEVELS>
+__global__ void __launch_bounds__(256, FMT == STF_FMT_F16 && C == 4 && !LEVELS ? 6 : 0) k_tex2d_cubic(Tex2DView t, LookupArgs a) {
+  using Parts = CubicParts<LEVELS>;
   constexpr uint32_t full = 0xffffffffu;
   const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31, k = lane & 3;
-  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x;
-  if (C * (FMT == STF_FMT_F32 ? 4 : 2) < 16 && a.lod != nullptr && t.levels > 1) {
-    tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
-    return;
-  }
-  {
-    // lanes whose neighbour's level-0 window is within a few texels of theirs
-    const float2 uv = first < n ? reinterpret_cast<const float2*>(a.coords)[first] : make_float2(0.0f, 0.0f);
-    const float x = uv.x * (float)t.level_w[0], y = uv.y * (float)t.level_h[0];
-    const float dx = __shfl_xor_sync(full, x, 1) - x, dy = __shfl_xor_sync(full, y, 1) - y;
-    if (__popc(__ballot_sync(full, fabsf(dx) < 5.0f && fabsf(dy) < 2.0f)) >= 16) {
-      tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
-      return;
-    }
-  }
   // (every lane of a warp runs the same iterations)
-  for (uint32_t i0 = first - lane; i0 < n; i0 += stride) {
+  for (uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += stride) {
     const uint32_t i = i0 + lane;
     const bool live = i < n;
     const float2 uv = live ? reinterpret_cast<const float2*>(a.coords)[i] : make_float2(0.0f, 0.0f);
     const float lod = live && a.lod ? a.lod[i] : 0.0f;
-    const DetLevels d = det_levels(t, a, lod);
-    const RasterPos p(t, d.L0, uv, live && d.w0 > 0.0f);
-    const RasterPos p1(t, d.L1, uv, live && d.w1 > 0.0f);
-    const bool blend = __any_sync(full, p1.on);
+    const Parts q(t, a, uv, lod, live);
+    // lanes whose neighbour's level-0 window is within a few texels of theirs
+    const float x0 = uv.x * (float)t.level_w[0], y0 = uv.y * (float)t.level_h[0];
+    const float dx = __shfl_xor_sync(full, x0, 1) - x0, dy = __shfl_xor_sync(full, y0, 1) - y0;
+    if (__popc(__ballot_sync(full, fabsf(dx) < 5.0f && fabsf(dy) < 2.0f)) >= 16) {
+      float v[4][C];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < C; ++c) v[j][c] = 0.0f;
+#pragma unroll
+      for (int p = 0; p < Parts::N; ++p) {
+        if (q.L[p] < 0) continue;
+        const CubicWindow<F, FMT, C> w(t, LEVELS ? q.L[p] : 0, q.x[p], q.y[p], q.w[p]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w.column(t, (j == 1 ? 2 : j == 2 ? 1 : j), v[(j == 1 ? 2 : j == 2 ? 1 : j)]);
+      }
+#pragma unroll
+      for (int c = 0; c < C; ++c) v[0][c] = (v[0][c] + v[2][c]) + (v[1][c] + v[3][c]);
+      if (!live) continue;
+      store_out<C>(a.out, i, v[0]);
+      continue;
+    }
+    const bool blend = LEVELS && __any_sync(full, q.L[Parts::N - 1] >= 0);
 #pragma unroll 1
     for (int r = 0; r < 4; ++r) {
       const int src = 8 * r + (lane >> 2);
       float v[C];
 #pragma unroll
       for (int c = 0; c < C; ++c) v[c] = 0.0f;
-      {
-        const float x = __shfl_sync(full, p.x[0], src), y = __shfl_sync(full, p.x[1], src);
-        const float sc = __shfl_sync(full, d.w0, src);
-        const int L = __shfl_sync(full, p.on ? p.L : -1, src);
-        if (L >= 0) tex2d_det_column<F, FMT, C>(t, L, x, y, sc, k, v);
-      }
-      if (blend) {
-        const float x = __shfl_sync(full, p1.x[0], src), y = __shfl_sync(full, p1.x[1], src);
-        const float sc = __shfl_sync(full, d.w1, src);
-        const int L = __shfl_sync(full, p1.on ? p1.L : -1, src);
-        if (L >= 0) tex2d_det_column<F, FMT, C>(t, L, x, y, sc, k, v);
+#pragma unroll
+      for (int p = 0; p < Parts::N; ++p) {
+        if (p == 1 && !blend) break;
+        const float x = __shfl_sync(full, q.x[p], src), y = __shfl_sync(full, q.y[p], src);
+        const float sc = LEVELS ? __shfl_sync(full, q.w[p], src) : 1.0f;
+        const int L = __shfl_sync(full, q.L[p], src);
+        if (L >= 0) CubicWindow<F, FMT, C>(t, LEVELS ? L : 0, x, y, sc).column(t, k, v);
       }
       // sum over the four lanes; each exchange halves the channels a lane keeps
       int c0 = 0;
@@ -595,6 +615,19 @@ __global__ void __launch_bounds__(256) k_tex2d_cubic(Tex2DView t, LookupArgs a) 
     }
   }
 }
+
+// The other cubic lookups of at most kFastLoopMaxQueries: one thread per query.
+template <int F, int FMT, int C>
+__global__ void __launch_bounds__(256) k_tex2d_cubic_each(Tex2DView t, LookupArgs a) {
+  tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
+}
+
+// Whether warps with levels of detail may take their queries by columns: texels of 16 bytes
+// and more.
+template <int FMT, int C>
+struct CubicLevels {
+  static constexpr bool value = C * (FMT == STF_FMT_F32 ? 4 : 2) >= 16;
+};
 
 template <int F, int FMT, int C>
 __global__ void __launch_bounds__(256) k_tex2d_deterministic(Tex2DView t, LookupArgs a) {
@@ -712,7 +745,10 @@ static cudaError_t run_tex2d(Op op, const Tex2DView& t, const LookupArgs& a, cud
         if (b.lod) b.lod += i;
         b.out += C * i;
         b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
-        k_tex2d_cubic<D, FMT, C><<<grid_blocks(b.n, threads), threads, 0, s>>>(t, b);
+        const int grid = grid_blocks(b.n, threads);
+        if (a.lod == nullptr || t.levels <= 1) k_tex2d_cubic<D, FMT, C, false><<<grid, threads, 0, s>>>(t, b);
+        else if constexpr (CubicLevels<FMT, C>::value) k_tex2d_cubic<D, FMT, C, true><<<grid, threads, 0, s>>>(t, b);
+        else k_tex2d_cubic_each<D, FMT, C><<<grid, threads, 0, s>>>(t, b);
       }
     }
     else k_tex2d_deterministic<D, FMT, C><<<blocks, threads, 0, s>>>(t, a);

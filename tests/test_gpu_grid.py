@@ -473,3 +473,26 @@ def test_cubic_scattered_and_neighbouring_warps(fmt, channels):
             # float32 means, within 2^-23 of the oracle's (and one binary16 rounding step)
             lim = 2e-6 * 1.25 ** 2 + (2.0 ** -11 if fmt == stf.FMT_F16 and l is not None else 0.0)
             assert np.all(np.abs(det - dv) <= lim)
+
+
+@pytest.mark.parametrize("fmt,channels", [(stf.FMT_F32, 1), (stf.FMT_F32, 4), (stf.FMT_F16, 2), (stf.FMT_F16, 4), (stf.FMT_F16, 8)])
+@pytest.mark.parametrize("filt", ["bspline3", "catmull_rom"])
+@pytest.mark.parametrize("levels", [1, 7])
+def test_cubic_values_do_not_depend_on_the_neighbouring_queries(fmt, channels, filt, levels):
+    """A query has the same bits among scattered queries, beside a copy of itself (a warp of
+    neighbours), in a part of the batch, and in a call that changes over half way."""
+    T = stf.Texture(stf.KIND_TEX2D, synth.texture2d(64, 64, channels, seed=3), dims=(64, 64, 1), channels=channels,
+                    fmt=fmt, mip_levels=levels, generate_mips=levels > 1)
+    n = 5003
+    uv = to_dev((synth.uniform(2 * n, 8).reshape(-1, 2) * np.float32(1.2) - np.float32(0.1)).astype(np.float32))
+    lod = None if levels == 1 else to_dev((synth.uniform(n, 9) * np.float32(8) - np.float32(1)).astype(np.float32))
+    def look(c, l):
+        return T.lookup_deterministic(c.contiguous(), None if l is None else l.contiguous(), filter=filt)
+    alone = look(uv, lod)
+    twice = look(uv.repeat_interleave(2, 0), None if lod is None else lod.repeat_interleave(2))
+    for k in (0, 1):
+        torch.testing.assert_close(twice[k::2], alone, rtol=0, atol=0)
+    torch.testing.assert_close(look(uv[17:], None if lod is None else lod[17:]), alone[17:], rtol=0, atol=0)
+    both = look(torch.cat([uv, uv.repeat_interleave(2, 0)]), None if lod is None else torch.cat([lod, lod.repeat_interleave(2)]))
+    torch.testing.assert_close(both[:n], alone, rtol=0, atol=0)
+    torch.testing.assert_close(both[n::2], alone, rtol=0, atol=0)
