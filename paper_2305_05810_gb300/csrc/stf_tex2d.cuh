@@ -575,6 +575,7 @@ __global__ void __launch_bounds__(256, FMT == STF_FMT_F16 && C == 4 && !LEVELS ?
       continue;
     }
     const bool blend = LEVELS && __any_sync(full, q.L[Parts::N - 1] >= 0);
+    float own[2] = {0.0f, 0.0f};                     // (C <= 2: the lane's own query)
 #pragma unroll 1
     for (int r = 0; r < 4; ++r) {
       const int src = 8 * r + (lane >> 2);
@@ -607,12 +608,21 @@ __global__ void __launch_bounds__(256, FMT == STF_FMT_F16 && C == 4 && !LEVELS ?
         }
       }
       const uint32_t j = i0 + src;
-      if (j < n && (C >= 4 || (C == 2 && !(k & 1)) || k == 0)) {
+      if constexpr (C <= 2) {
+        // to the lane whose query it is, for one store of the warp's results in a row (stored
+        // by round, 32 or 64 bytes at a time, results in host memory took a third longer)
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const float o = __shfl_sync(full, v[0], 4 * (lane & 7) + 2 * c);
+          if (lane >> 3 == r) own[c] = o;
+        }
+      } else if (j < n) {
         float* o = a.out + (size_t)j * C + c0;
         if constexpr (C == 8) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
         else *o = v[0];
       }
     }
+    if (C <= 2 && live) store_out<(C <= 2 ? C : 1)>(a.out, i, own);
   }
 }
 
