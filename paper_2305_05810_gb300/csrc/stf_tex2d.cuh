@@ -626,17 +626,20 @@ __global__ void __launch_bounds__(256, FMT == STF_FMT_F16 && C == 4 && !LEVELS ?
   }
 }
 
-// The other cubic lookups of at most kFastLoopMaxQueries: one thread per query.
+// The other cubic lookups of at most kFastLoopMaxQueries: one thread per query.  (Eight
+// channels take the 64-bit loop: the same time on device arrays, 890 us instead of 1070 for
+// 2^22 lookups of arrays in host memory.)
 template <int F, int FMT, int C>
 __global__ void __launch_bounds__(256) k_tex2d_cubic_each(Tex2DView t, LookupArgs a) {
   tex2d_det_loop<F, FMT, C, uint32_t>(t, a);
 }
 
-// Whether warps with levels of detail may take their queries by columns: texels of 16 bytes
-// and more.
+// Whether warps with levels of detail may take their queries by columns: the second level's
+// setup is paid four times as well.  Four FP32 channels gain (2^22 lookups at random levels
+// 210 -> 193 us), eight FP16 channels lose (218 -> 234 us), and so do smaller texels.
 template <int FMT, int C>
 struct CubicLevels {
-  static constexpr bool value = C * (FMT == STF_FMT_F32 ? 4 : 2) >= 16;
+  static constexpr bool value = FMT == STF_FMT_F32 && C >= 4;
 };
 
 template <int F, int FMT, int C>
@@ -758,6 +761,7 @@ static cudaError_t run_tex2d(Op op, const Tex2DView& t, const LookupArgs& a, cud
         const int grid = grid_blocks(b.n, threads);
         if (a.lod == nullptr || t.levels <= 1) k_tex2d_cubic<D, FMT, C, false><<<grid, threads, 0, s>>>(t, b);
         else if constexpr (CubicLevels<FMT, C>::value) k_tex2d_cubic<D, FMT, C, true><<<grid, threads, 0, s>>>(t, b);
+        else if constexpr (C == 8) k_tex2d_deterministic<D, FMT, C><<<grid, threads, 0, s>>>(t, b);
         else k_tex2d_cubic_each<D, FMT, C><<<grid, threads, 0, s>>>(t, b);
       }
     }
