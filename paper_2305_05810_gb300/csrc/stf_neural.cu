@@ -16,6 +16,7 @@
 
 #include "stf_internal.h"
 #include "stf_memory.h"
+#include "stf_once.h"
 #include "stf_round.h"
 
 namespace stf {
@@ -1170,12 +1171,11 @@ __global__ void __launch_bounds__(128 * tct::GROUPS, 1) k_neural_train_tc(Neural
 // Forward, backward and parameter gradients of a batch (ta.grads and ta.loss zero before).
 static cudaError_t launch_train_tc(const NeuralDev& nd, const TrainArgs& ta, cudaStream_t s) {
   const int smem = (int)sizeof(tct::Smem);
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_neural_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t e = once([&] {
+    return cudaFuncSetAttribute(k_neural_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  });
+  if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1260,17 +1260,14 @@ __global__ void k_rows_to_h8(const float* src, int cin, __half* dst, int64_t row
 
 // Launches a decode kernel over `tiles` tiles, two per CTA pass.
 template <class Kernel>
-static cudaError_t launch_decode(Kernel k, bool& ready, int64_t tiles, const NeuralDev& nd, const LookupArgs& a,
+static cudaError_t launch_decode(Kernel k, OncePerDevice& once, int64_t tiles, const NeuralDev& nd, const LookupArgs& a,
                                  cudaStream_t s) {
   // at least 46 KiB of shared memory per CTA keeps at most 4 CTAs on an SM (228 KiB),
   // so their 4 x 128 tensor-memory columns fit in the SM's 512 and no allocation waits
   const int need = (int)sizeof(tc::Smem) + 1024;
   const int smem = need > 46 * 1024 ? need : 46 * 1024;
-  if (!ready) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    ready = true;
-  }
+  const cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+  if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1282,17 +1279,17 @@ static cudaError_t launch_decode(Kernel k, bool& ready, int64_t tiles, const Neu
 
 template <int F>
 static cudaError_t run_neural(Op op, const NeuralDev& nd, const LookupArgs& a, cudaStream_t s) {
-  static bool ready[3];
+  static OncePerDevice once[3];
   const int64_t tiles = (a.n + tc::ROWS - 1) / tc::ROWS;
   if (op == OP_STOCHASTIC) {
     if (a.perm == nullptr && a.taps == nullptr)
-      return launch_decode(k_neural_stochastic_tc<F, true>, ready[0], tiles, nd, a, s);
-    return launch_decode(k_neural_stochastic_tc<F, false>, ready[1], tiles, nd, a, s);
+      return launch_decode(k_neural_stochastic_tc<F, true>, once[0], tiles, nd, a, s);
+    return launch_decode(k_neural_stochastic_tc<F, false>, once[1], tiles, nd, a, s);
   }
   if (op == OP_DETERMINISTIC) {
     const int parts = (a.lod != nullptr && nd.nlev > 1 && a.level_mode != STF_LEVEL_NEAREST) ? 2 : 1;
     const int q = tc::ROWS / (parts * Filter<F>::T * Filter<F>::T);
-    return launch_decode(k_neural_deterministic_tc<F>, ready[2], (a.n + q - 1) / q, nd, a, s);
+    return launch_decode(k_neural_deterministic_tc<F>, once[2], (a.n + q - 1) / q, nd, a, s);
   }
   return cudaErrorNotSupported;
 }
