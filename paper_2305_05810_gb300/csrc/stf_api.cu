@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "stf_internal.h"
+#include "stf_memory.h"
 
 namespace {
 
@@ -77,6 +78,8 @@ int grid_blocks(int64_t n, int threads, int waves) {
 int queue_blocks(int64_t n, int threads, int per_sm) {
   return capped_blocks(n, threads, (int64_t)sm_count() * per_sm);
 }
+
+bool local_arrays(const LookupArgs& a) { return local_memory(a.out) && local_memory(a.coords); }
 
 bool handle_ok(stf_texture t) {
   std::lock_guard<std::mutex> lk(g_registry_mutex);

@@ -139,24 +139,22 @@ __global__ void __launch_bounds__(256, dense_stochastic_min_blocks<F>()) k_dense
       return;
     }
   }
-  if constexpr (!FixedWindow<F>::value || REUSE) {   // (the others went by queue)
-    if (off32 && quad_loop3_ok(a)) {
-      quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
-        float x[3] = {x0, x1, x2};
-        int4 tap;
-        return dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, j, a.sample_index, tap, &mb);
-      });
-      return;
+  if (off32 && quad_loop3_ok(a)) {
+    quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
+      float x[3] = {x0, x1, x2};
+      int4 tap;
+      return dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, j, a.sample_index, tap, &mb);
+    });
+    return;
+  }
+  if (fast_loop(a) && off32) {
+    const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+      float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
+      int4 tap;
+      a.out[i] = dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, i, a.sample_index, tap, &mb);
     }
-    if (fast_loop(a) && off32) {
-      const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
-      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
-        int4 tap;
-        a.out[i] = dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, i, a.sample_index, tap, &mb);
-      }
-      return;
-    }
+    return;
   }
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
@@ -362,6 +360,33 @@ __global__ void __launch_bounds__(256, kDenseDetBlocks) k_dense_deterministic(De
   }
 }
 
+// One thread per query, for arrays that are not in this device's memory, whose link bounds the
+// call: a queued kernel writes results twice and reads coordinates from few warps (4 M hits with
+// results in host memory, trilinear 96 us in place, 514 us queued; tricubic 258 and 590 us).
+template <int F, int FMT>
+__global__ void __launch_bounds__(256) k_dense_deterministic_each(Dense3DView g, LookupArgs a) {
+  constexpr int T = Filter<F>::T, OFF0 = Filter<F>::OFF0;
+  __shared__ LiveBox live, inner;
+  const bool off32 = (uint64_t)g.nx * (uint64_t)g.ny * (uint64_t)g.nz <= (uint64_t(1) << 32);
+  if (threadIdx.x == 0) {
+    const int zero[3] = {0, 0, 0}, dims[3] = {g.nx, g.ny, g.nz};
+    live = live_box(zero, dims, OFF0, OFF0 + T - 1);
+    inner = live_box(zero, dims, OFF0 + T - 1, OFF0);
+  }
+  __syncthreads();
+  const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
+    float acc = g.background;
+    if (live.has(x)) {
+      const bool in = off32 && inner.has(x);
+      prepare_coords<3>(x);
+      acc = in ? dense_inner_sum<F, FMT>(g, x) : dense_edge_sum<F, FMT>(g, x);
+    }
+    a.out[i] = acc;
+  }
+}
+
 // Deterministic form of the Gaussian FIS filter: one thread per query.
 template <int FMT>
 __global__ void __launch_bounds__(256) k_dense_gaussian(Dense3DView g, LookupArgs a) {
@@ -410,7 +435,8 @@ static cudaError_t run_dense(Op op, const Dense3DView& g, const LookupArgs& a, c
   if (op == OP_STOCHASTIC) {
     if constexpr (FixedWindow<F>::value) {
       const bool off32 = (uint64_t)g.nx * (uint64_t)g.ny * (uint64_t)g.nz <= (uint64_t(1) << 32);
-      if (off32 && fast_loop(a) && !(UsesReuse<F>::value && a.reuse)) {
+      // (results in host memory, which the queue writes twice: in place, 4 M hits 96 us, 495 queued)
+      if (off32 && fast_loop(a) && !(UsesReuse<F>::value && a.reuse) && local_arrays(a)) {
         if (a.n >= kQueueChunkMin)
           k_dense_stochastic_queue<F, FMT, 4><<<queue_blocks((a.n + 3) / 4, threads, kDenseQueueBlocks), threads, 0, s>>>(g, a);
         else
@@ -435,10 +461,13 @@ static cudaError_t run_dense(Op op, const Dense3DView& g, const LookupArgs& a, c
         b.coords += 3 * i;
         b.out += i;
         b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
-        if (b.n >= kQueueChunkMin)
+        if (!local_arrays(a)) {
+          k_dense_deterministic_each<D, FMT><<<grid_blocks(b.n, threads), threads, 0, s>>>(g, b);
+        } else if (b.n >= kQueueChunkMin) {
           k_dense_deterministic<D, FMT, 4><<<queue_blocks((b.n + 3) / 4, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
-        else
+        } else {
           k_dense_deterministic<D, FMT, 1><<<queue_blocks(b.n, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
+        }
       }
     }
   } else {

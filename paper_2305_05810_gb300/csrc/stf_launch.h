@@ -26,6 +26,10 @@ constexpr int kStochasticWaves = 8;
 // call over more warps.
 constexpr int64_t kQueueChunkMin = 1 << 20;
 
+// Whether a call's coordinates and results lie in this device's memory.  Queued 3D kernels need
+// that: across a link, few warps read ahead too little, and results are written twice.
+bool local_arrays(const LookupArgs& a);
+
 // The filter whose deterministic form filter F has.
 constexpr int deterministic_filter(int F) {
   return F == STF_FILTER_FIS_LINEAR ? STF_FILTER_LINEAR

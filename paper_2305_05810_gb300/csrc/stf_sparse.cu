@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "stf_internal.h"
+#include "stf_memory.h"
 
 namespace stf {
 
@@ -379,24 +380,22 @@ __global__ void __launch_bounds__(256) k_sparse_stochastic(SparseDev g, LookupAr
   __shared__ UpperSmem su;
   stage_upper(g, su);
   const MissBox mb = miss_box<F>(g.bb_lo[0], g.bb_lo[1], g.bb_lo[2], g.bb_hi[0], g.bb_hi[1], g.bb_hi[2]);
-  if constexpr (!FixedWindow<F>::value || REUSE) {   // (the others went by queue)
-    if (quad_loop3_ok(a)) {
-      quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
-        float x[3] = {x0, x1, x2};
-        int4 tap;
-        return sparse_stochastic_at<F, FMT, REUSE>(g, su, a, x, j, a.sample_index, tap, &mb);
-      });
-      return;
+  if (quad_loop3_ok(a)) {
+    quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
+      float x[3] = {x0, x1, x2};
+      int4 tap;
+      return sparse_stochastic_at<F, FMT, REUSE>(g, su, a, x, j, a.sample_index, tap, &mb);
+    });
+    return;
+  }
+  if (fast_loop(a)) {
+    const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+      float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
+      int4 tap;
+      a.out[i] = sparse_stochastic_at<F, FMT, REUSE>(g, su, a, x, i, a.sample_index, tap, &mb);
     }
-    if (fast_loop(a)) {
-      const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
-      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
-        int4 tap;
-        a.out[i] = sparse_stochastic_at<F, FMT, REUSE>(g, su, a, x, i, a.sample_index, tap, &mb);
-      }
-      return;
-    }
+    return;
   }
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
@@ -496,14 +495,14 @@ struct SparseQueue {
   int32_t leaf[8][TAPS];                        // by corner: bits 0, 1, 2 the next leaf along x, y, z
 };
 
-// Filtered value from the leaves in queue slot s.  Taps are summed along z (contiguous in
-// a leaf) in a column, then the columns weighted by wx * wy.
-template <int F, int FMT>
-__device__ __forceinline__ float sparse_window_sum(const SparseDev& g, const SparseQueue& q, int s) {
+// Filtered value at (x0, x1, x2) from the window's leaves, leaf(corner).  Taps are summed along
+// z (contiguous in a leaf) in a column, then the columns weighted by wx * wy.
+template <int F, int FMT, class Leaf>
+__device__ __forceinline__ float sparse_window_sum(const SparseDev& g, float x0, float x1, float x2, Leaf leaf) {
   using Fl = Filter<F>;
   float fx, fy, fz;
-  const int bx = axis_base(q.tap_x[0][s], fx) + Fl::OFF0, by = axis_base(q.tap_x[1][s], fy) + Fl::OFF0,
-            bz = axis_base(q.tap_x[2][s], fz) + Fl::OFF0;
+  const int bx = axis_base(x0, fx) + Fl::OFF0, by = axis_base(x1, fy) + Fl::OFF0,
+            bz = axis_base(x2, fz) + Fl::OFF0;
   float wx[Fl::T], wy[Fl::T], wz[Fl::T];
   Fl::weights(fx, wx);
   Fl::weights(fy, wy);
@@ -521,7 +520,7 @@ __device__ __forceinline__ float sparse_window_sum(const SparseDev& g, const Spa
     for (int kx = 0; kx < Fl::T; ++kx) {
       const int x = bx + kx, sx = (x >> 3) != (bx >> 3);
       const int c = (sy << 1) | sx, column = ((x & 7) << 6) | ((y & 7) << 3);
-      const int la = q.leaf[c][s], lb = q.leaf[4 | c][s];   // lb is used past z = 7 only
+      const int la = leaf(c), lb = leaf(4 | c);   // lb is used past z = 7 only
       float v[Fl::T];
       if constexpr (FMT == STF_FMT_F32) {
         const float* pa = g.leaf_f32 + ((int64_t)la * 512 + column + z);
@@ -623,12 +622,44 @@ __global__ void __launch_bounds__(256, kSparseDetBlocks) k_sparse_deterministic(
       if (n_taps >= (more || n_box > 0 ? 32 : 1)) {
         const uint32_t count = min(n_taps, 32u);
         n_taps -= count;
-        if (lane < count) a.out[q.tap_i[n_taps + lane]] = sparse_window_sum<F, FMT>(g, q, n_taps + lane);
+        const uint32_t s = n_taps + lane;
+        if (lane < count)
+          a.out[q.tap_i[s]] = sparse_window_sum<F, FMT>(g, q.tap_x[0][s], q.tap_x[1][s], q.tap_x[2][s],
+                                                        [&](int c) { return q.leaf[c][s]; });
         __syncwarp();
       }
     }
     if (!more) break;
     __syncwarp();          // the slots just read may be filled again
+  }
+}
+
+// The same one thread per query, for arrays that are not in this device's memory (as in
+// k_dense_deterministic_each).
+template <int F, int FMT>
+__global__ void __launch_bounds__(256) k_sparse_deterministic_each(SparseDev g, LookupArgs a) {
+  using Fl = Filter<F>;
+  __shared__ UpperSmem su;
+  __shared__ LiveBox live;
+  if (threadIdx.x == 0) live = live_box(g.bb_lo, g.bb_hi, Fl::OFF0, Fl::OFF0 + Fl::T - 1);
+  stage_upper(g, su);                                // (ends with a barrier)
+  const uint32_t n = (uint32_t)a.n, stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
+    float acc = g.background;
+    if (live.has(x)) {
+      int leaf[8];
+      prepare_coords<3>(x);
+      if (sparse_window_leaves<Fl::T>(g, su, (int)floorf(x[0]) + Fl::OFF0, (int)floorf(x[1]) + Fl::OFF0,
+                                      (int)floorf(x[2]) + Fl::OFF0, leaf))
+        acc = sparse_window_sum<F, FMT>(g, x[0], x[1], x[2], [&](int c) {
+          int l = leaf[0];
+#pragma unroll
+          for (int k = 1; k < 8; ++k) l = c == k ? leaf[k] : l;
+          return l;
+        });
+    }
+    a.out[i] = acc;
   }
 }
 
@@ -676,7 +707,9 @@ static cudaError_t run_sparse(Op op, const SparseDev& g, const LookupArgs& a, cu
   const int blocks = grid_blocks(units, threads, op == OP_STOCHASTIC ? kStochasticWaves : 4);
   if (op == OP_STOCHASTIC) {
     if constexpr (FixedWindow<F>::value) {
-      if (fast_loop(a) && !(UsesReuse<F>::value && a.reuse)) {
+      // (results in host memory, written twice by queue: in place, unless the coordinates, which
+      // the queue loads ahead, come across the link as well: 14.7 M samples 580 us by queue, 685)
+      if (fast_loop(a) && !(UsesReuse<F>::value && a.reuse) && (local_memory(a.out) || !local_memory(a.coords))) {
         if (a.n >= kQueueChunkMin)
           k_sparse_stochastic_queue<F, FMT, 4><<<queue_blocks((a.n + 3) / 4, threads, kSparseQueueBlocks), threads, 0, s>>>(g, a);
         else
@@ -701,7 +734,9 @@ static cudaError_t run_sparse(Op op, const SparseDev& g, const LookupArgs& a, cu
         b.coords += 3 * i;
         b.out += i;
         b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
-        if (b.n >= kQueueChunkMin)
+        if (!local_arrays(a))
+          k_sparse_deterministic_each<D, FMT><<<grid_blocks(b.n, threads), threads, 0, s>>>(g, b);
+        else if (b.n >= kQueueChunkMin)
           k_sparse_deterministic<D, FMT, 4><<<queue_blocks((b.n + 3) / 4, threads, kSparseDetBlocks), threads, 0, s>>>(g, b);
         else
           k_sparse_deterministic<D, FMT, 1><<<queue_blocks(b.n, threads, kSparseDetBlocks), threads, 0, s>>>(g, b);

@@ -154,3 +154,27 @@ def test_stochastic_queue_equals_the_general_loop(kind, filt):
             want = T.lookup(c, taps=torch.empty((n, 4), dtype=torch.int32, device=dev()), **args)
             torch.testing.assert_close(out[shift:shift + n], want, rtol=0, atol=0)
             assert float(out[0 if shift else n]) == 7.0
+
+
+@pytest.mark.parametrize("filt", ["linear", "bspline3"])
+@pytest.mark.parametrize("kind", ["dense", "sparse"])
+def test_arrays_in_host_memory_give_the_same_bits(kind, filt):
+    """Coordinates, results or both in page-locked memory, which take the kernels without a
+    queue."""
+    T, _ = _dense(stf.FMT_F16) if kind == "dense" else _sparse(stf.FMT_E4M3_SCALED)
+    for n in (33, 4099, CHUNKED + 77):
+        p = _points(n, 0, 23, 5) if kind == "dense" else _points(n, -32, 32, 5) + np.array([128, 0, 4096], np.float32)
+        c = to_dev(p.astype(np.float32))
+        host = torch.empty((n, 3), pin_memory=True)
+        host.copy_(c)
+        for look in (lambda x, out=None: T.lookup_deterministic(x, filter=filt, out=out),
+                     lambda x, out=None: T.lookup(x, filter=filt, seed=3, out=out)):
+            want = look(c)
+            out = torch.full((n, 1), 7.0, device=dev())
+            look(host, out)
+            torch.testing.assert_close(out, want, rtol=0, atol=0)
+            for x in (c, host):
+                out = torch.full((n, 1), 7.0, pin_memory=True)
+                look(x, out)
+                stf.stf_synchronize(T.handle)
+                torch.testing.assert_close(out, want.cpu(), rtol=0, atol=0)
