@@ -360,9 +360,11 @@ __global__ void __launch_bounds__(256, kDenseDetBlocks) k_dense_deterministic(De
   }
 }
 
-// One thread per query, for arrays that are not in this device's memory, whose link bounds the
-// call: a queued kernel writes results twice and reads coordinates from few warps (4 M hits with
-// results in host memory, trilinear 96 us in place, 514 us queued; tricubic 258 and 590 us).
+// One thread per query: the trilinear filter (eight scattered voxels: 14.7 M ray-march samples
+// of a 256^3 FP16 grid 100 us in place, 115 us queued; 4 M hits 72 and 84 us), and arrays that
+// are not in this device's memory, whose link bounds the call: a queued kernel writes results
+// twice and reads coordinates from few warps (4 M hits with results in host memory, trilinear
+// 96 us in place, 514 us queued; tricubic 258 and 590 us).
 template <int F, int FMT>
 __global__ void __launch_bounds__(256) k_dense_deterministic_each(Dense3DView g, LookupArgs a) {
   constexpr int T = Filter<F>::T, OFF0 = Filter<F>::OFF0;
@@ -379,7 +381,7 @@ __global__ void __launch_bounds__(256) k_dense_deterministic_each(Dense3DView g,
     float x[3] = {__ldg(a.coords + 3 * i), __ldg(a.coords + 3 * i + 1), __ldg(a.coords + 3 * i + 2)};
     float acc = g.background;
     if (live.has(x)) {
-      const bool in = off32 && inner.has(x);
+      const bool in = T == 4 && off32 && inner.has(x);
       prepare_coords<3>(x);
       acc = in ? dense_inner_sum<F, FMT>(g, x) : dense_edge_sum<F, FMT>(g, x);
     }
@@ -461,13 +463,16 @@ static cudaError_t run_dense(Op op, const Dense3DView& g, const LookupArgs& a, c
         b.coords += 3 * i;
         b.out += i;
         b.n = a.n - i < kFastLoopMaxQueries ? a.n - i : kFastLoopMaxQueries;
-        if (!local_arrays(a)) {
-          k_dense_deterministic_each<D, FMT><<<grid_blocks(b.n, threads), threads, 0, s>>>(g, b);
-        } else if (b.n >= kQueueChunkMin) {
-          k_dense_deterministic<D, FMT, 4><<<queue_blocks((b.n + 3) / 4, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
-        } else {
-          k_dense_deterministic<D, FMT, 1><<<queue_blocks(b.n, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
+        if constexpr (Filter<D>::T == 4) {
+          if (local_arrays(a)) {
+            if (b.n >= kQueueChunkMin)
+              k_dense_deterministic<D, FMT, 4><<<queue_blocks((b.n + 3) / 4, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
+            else
+              k_dense_deterministic<D, FMT, 1><<<queue_blocks(b.n, threads, kDenseDetBlocks), threads, 0, s>>>(g, b);
+            continue;
+          }
         }
+        k_dense_deterministic_each<D, FMT><<<grid_blocks(b.n, threads), threads, 0, s>>>(g, b);
       }
     }
   } else {
