@@ -95,13 +95,23 @@ template <int F, int FMT, int PER>
 __global__ void __launch_bounds__(256, kDenseQueueBlocks) k_dense_stochastic_queue(Dense3DView g, LookupArgs a) {
   using W = FixedWindow<F>;
   __shared__ LiveQueue<PER> queues[8];
-  __shared__ LiveBox live;
-  if (threadIdx.x == 0) {
-    const int zero[3] = {0, 0, 0}, dims[3] = {g.nx, g.ny, g.nz};
-    live = live_box(zero, dims, W::LO, W::HI);
-  }
+  __shared__ LiveCall call;
+  const int zero[3] = {0, 0, 0}, dims[3] = {g.nx, g.ny, g.nz};
+  stage_live<PER>(a, live_box(zero, dims, W::LO, W::HI), call);
   __syncthreads();
-  live_queue_loop<PER>(a, g.background, live, queues[threadIdx.x >> 5], [&](uint32_t i, float (&x)[3], bool ok) {
+  if (PER == 4 && call.direct) {
+    const MissBox mb = miss_box<F>(0, 0, 0, g.nx, g.ny, g.nz);
+    quad_loop3_joint(a, [&](float (&x)[4][3], uint32_t i) {
+      return joint_one_tap4<F>(a, x, i, mb, g.background,
+                               [&](const int* t) { return dense_fetch<FMT, true>(g, t[0], t[1], t[2]); });
+    }, [&](float x0, float x1, float x2, uint32_t j) {
+      float x[3] = {x0, x1, x2};
+      int4 tap;
+      return dense_stochastic_at<F, FMT, false, true>(g, a, x, j, a.sample_index, tap, &mb);
+    });
+    return;
+  }
+  live_queue_loop<PER>(a, g.background, call.box, queues[threadIdx.x >> 5], [&](uint32_t i, float (&x)[3], bool ok) {
     const uint4 v = query_variates(a, i, a.sample_index);
     prepare_coords<3>(x);
     int t[3];
@@ -140,7 +150,7 @@ __global__ void __launch_bounds__(256, dense_stochastic_min_blocks<F>()) k_dense
     }
   }
   if (off32 && quad_loop3_ok(a)) {
-    quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
+    quad_loop3(a, (uint32_t)a.n >> 2, [&](float x0, float x1, float x2, uint32_t j) {
       float x[3] = {x0, x1, x2};
       int4 tap;
       return dense_stochastic_at<F, FMT, REUSE, true>(g, a, x, j, a.sample_index, tap, &mb);

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(256) k_sparse_stochastic(SparseDev g, LookupAr
   stage_upper(g, su);
   const MissBox mb = miss_box<F>(g.bb_lo[0], g.bb_lo[1], g.bb_lo[2], g.bb_hi[0], g.bb_hi[1], g.bb_hi[2]);
   if (quad_loop3_ok(a)) {
-    quad_loop3(a, [&](float x0, float x1, float x2, uint32_t j) {
+    quad_loop3(a, (uint32_t)a.n >> 2, [&](float x0, float x1, float x2, uint32_t j) {
       float x[3] = {x0, x1, x2};
       int4 tap;
       return sparse_stochastic_at<F, FMT, REUSE>(g, su, a, x, j, a.sample_index, tap, &mb);
@@ -417,10 +417,21 @@ __global__ void __launch_bounds__(256, kSparseQueueBlocks) k_sparse_stochastic_q
   using W = FixedWindow<F>;
   __shared__ UpperSmem su;
   __shared__ LiveQueue<PER> queues[8];
-  __shared__ LiveBox live;
-  if (threadIdx.x == 0) live = live_box(g.bb_lo, g.bb_hi, W::LO, W::HI);
+  __shared__ LiveCall call;
+  stage_live<PER>(a, live_box(g.bb_lo, g.bb_hi, W::LO, W::HI), call);
   stage_upper(g, su);                                // (ends with a barrier)
-  live_queue_loop<PER>(a, g.background, live, queues[threadIdx.x >> 5], [&](uint32_t i, float (&x)[3], bool ok) {
+  if (PER == 4 && call.direct) {
+    const MissBox mb = miss_box<F>(g.bb_lo[0], g.bb_lo[1], g.bb_lo[2], g.bb_hi[0], g.bb_hi[1], g.bb_hi[2]);
+    // (whole rounds of four; a last round for some threads only would hold up the rest)
+    const uint32_t groups = (uint32_t)a.n >> 2;
+    quad_loop3(a, groups - groups % (gridDim.x * blockDim.x), [&](float x0, float x1, float x2, uint32_t j) {
+      float x[3] = {x0, x1, x2};
+      int4 tap;
+      return sparse_stochastic_at<F, FMT, false>(g, su, a, x, j, a.sample_index, tap, &mb);
+    });
+    return;
+  }
+  live_queue_loop<PER>(a, g.background, call.box, queues[threadIdx.x >> 5], [&](uint32_t i, float (&x)[3], bool ok) {
     const uint4 v = query_variates(a, i, a.sample_index);
     prepare_coords<3>(x);
     int t[3];

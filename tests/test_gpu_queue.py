@@ -178,3 +178,23 @@ def test_arrays_in_host_memory_give_the_same_bits(kind, filt):
                 look(x, out)
                 stf.stf_synchronize(T.handle)
                 torch.testing.assert_close(out, want.cpu(), rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("filt", ["linear", "bspline3", "fis_bspline3"])
+@pytest.mark.parametrize("kind", ["dense", "sparse"])
+def test_calls_taken_directly_and_by_queue(kind, filt):
+    """Calls of whose queries three quarters are live are taken without the queue, judged by a
+    few of them: the same bits for any share and place of the live ones."""
+    T, _ = _dense(stf.FMT_F16) if kind == "dense" else _sparse(stf.FMT_E4M3_SCALED)
+    for n in (CHUNKED, CHUNKED + 77):
+        i, u = np.arange(n), synth.uniform(n, 6)
+        p = synth.uniform(3 * n, 5).reshape(-1, 3) * np.float32(14)
+        p += np.float32(4) if kind == "dense" else np.array([124, -4, 4092], np.float32)
+        for live in (i >= 0, u < 0.8, u < 0.75, u < 0.7, i < n // 2, i >= n // 2, i % 128 < 100):
+            x = p.copy()
+            x[~live] = -1e5
+            x[::1001] = np.nan
+            c = to_dev(x)
+            args = dict(filter=filt, seed=11, query_offset=(1 << 32) - 1000)
+            want = T.lookup(c, taps=torch.empty((n, 4), dtype=torch.int32, device=dev()), **args)
+            torch.testing.assert_close(T.lookup(c, **args), want, rtol=0, atol=0)
