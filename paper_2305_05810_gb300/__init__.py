@@ -155,7 +155,8 @@ def _stream(stream):
         import torch
         if torch.cuda.is_initialized():
             # the raw handle, without a Stream object and a device query: a small lookup's call
-            # is host time (65,536 points: 17.3 us a call with them and named structure fields, 12.7 us now)
+            # is host time (65,536 points: 19.6 us a pass with them and named structure fields,
+            # 17.1 us now, though runs of either differ by more)
             return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
     if isinstance(stream, int):

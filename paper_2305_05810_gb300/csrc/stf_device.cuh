@@ -675,25 +675,26 @@ __device__ __forceinline__ void pick_fis(const float* x, const LookupArgs& a, in
   }
 }
 
-// Filters whose dense 3D stochastic lookups take the joint four-query form: the Gaussian
-// (3% sooner than one query after another on the dense benchmark rays).  The fixed-window
-// filters go by queue; Catmull-Rom measured 4% slower in it and keeps the one-query form,
-// as do the two-tap positivized estimator and the sparse grids (7% slower).
+// Filters whose dense 3D stochastic lookups take the joint four-query form in
+// k_dense_stochastic: the Gaussian (3% sooner than one query after another on ray-march
+// samples).  The fixed-window filters take it in their own kernel, for calls that are mostly
+// live; Catmull-Rom measured 4% slower in it and keeps the one-query form, as do the two-tap
+// positivized estimator and the sparse grids (7% slower).
 template <int F, bool REUSE>
 struct JointOneTap {
   static constexpr bool value = F == STF_FILTER_FIS_GAUSSIAN && !REUSE;
 };
 
 // The tap of one such lookup at coordinates x (checked by prepare_coords) from its
-// stream-0 variates r; returns the estimator's scale (sign * S for Catmull-Rom, else 1).
+// stream-0 variates r.
 template <int F>
-__device__ __forceinline__ float draw_one_tap3(const LookupArgs& a, const float* x, uint32_t j,
+__device__ __forceinline__ void draw_one_tap3(const LookupArgs& a, const float* x, uint32_t j,
                                                const uint4& r, int* idx) {
   if constexpr (IsFis<F>::value) {
     pick_fis<F, 3>(x, a, j, a.sample_index, r, idx);
-    return 1.0f;
   } else {
-    return pick_taps_r<F, 3, false>(x, r, idx);
+    static_assert(Filter<F>::NONNEG, "a tap without a scale");
+    pick_taps_r<F, 3, false>(x, r, idx);
   }
 }
 
@@ -721,17 +722,11 @@ __device__ __forceinline__ float4 joint_one_tap4(const LookupArgs& a, float (&x)
 #pragma unroll
     for (int k = 0; k < 4; ++k) r[k] = query_variates(a, i + k, a.sample_index);
     int idx[4][3];
-    float sigma[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) sigma[k] = draw_one_tap3<F>(a, x[k], i + k, r[k], idx[k]);
+    for (int k = 0; k < 4; ++k) draw_one_tap3<F>(a, x[k], i + k, r[k], idx[k]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (live[k]) {
-        float t = fetch(idx[k]);
-        if constexpr (F == STF_FILTER_CATMULL_ROM) t *= sigma[k];
-        v[k] = t;
-      }
-    }
+    for (int k = 0; k < 4; ++k)
+      if (live[k]) v[k] = fetch(idx[k]);
   }
   return make_float4(v[0], v[1], v[2], v[3]);
 }

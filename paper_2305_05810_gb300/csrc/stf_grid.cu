@@ -2,7 +2,8 @@
 // kernels are in stf_tex2d.cuh, one translation unit per storage format), and the
 // create-time kernels of regular grids.
 //
-// One thread per query (grid-stride).  The stochastic kernels draw one tap per axis
+// One thread per query (grid-stride), or warps that queue the queries that need work (the
+// fixed-window filters).  The stochastic kernels draw one tap per axis
 // by inverse CDF over |w| (sampling arrays, Section 2.2; separable sampling,
 // Section 4.2) and fetch a single texel (Eq. 3); the deterministic kernels sum all
 // 2^d / 4^d taps (Eq. 2, Eq. 9); the accumulate kernels repeat the stochastic form
@@ -86,8 +87,8 @@ __device__ __forceinline__ float dense_stochastic_one(const Dense3DView& g, cons
 // grids of at most 2^32 voxels and at most kFastLoopMaxQueries queries, without tap output
 // or permutation.  A ray-march chunk holds from none to three quarters of live samples; the
 // queue lets every draw run on full lanes.  33 M samples of a 256^3 FP16 grid, B-spline:
-// 133 us with the live ones of each chunk packed on its own lanes (two or four draws a
-// lane), 117 us by queue (88 M instead of 117 M warp instructions; the coordinates kept
+// 135 us with the live ones of each chunk packed on its own lanes (two or four draws a
+// lane), 121 us by queue (95 M instead of 117 M warp instructions; the coordinates kept
 // beside the indices instead of read again: 4 us; the next chunk loaded ahead on five
 // blocks an SM instead of six: 3 us; two draws a lane: 3 us slower).
 constexpr int kDenseQueueBlocks = 5;      // resident 256-thread blocks per SM
@@ -121,8 +122,9 @@ __global__ void __launch_bounds__(256, kDenseQueueBlocks) k_dense_stochastic_que
 }
 
 // Resident 256-thread blocks per SM: six (at most 40 registers a thread) for the tent
-// and B-spline filters, 1.4% sooner than five on the dense benchmark call without
-// spills; five for Catmull-Rom and the Gaussian, which would spill at 40; four for
+// and B-spline filters, 1.4% sooner than five without spills when ray marches took this
+// kernel (now the other calls do: host memory, tap output, binned, one variate reused); five
+// for Catmull-Rom and the Gaussian, which would spill at 40; four for
 // the two-tap positivized Catmull-Rom (at 84 registers and three blocks it ran 17%
 // slower).
 template <int F>
@@ -306,9 +308,9 @@ constexpr int kDenseDetBlocks = 3;   // resident 256-thread blocks per SM
 // the others in shared memory; whenever 32 windows of one kind wait, they run on all 32
 // lanes.  Ray-march samples mix misses, inner and edge windows in every warp: run in
 // place, 10 of 32 lanes were active.  8.3 M samples of a 256^3 FP16 grid, tricubic:
-// 311 us in place, 168 us queued (75 M instead of 184 M warp instructions), now bound by
+// 323 us in place, 173 us queued (60 M instead of 184 M warp instructions), now bound by
 // the L1 wavefronts of the row loads (84%).  The grid is the resident blocks only: with
-// two waves of blocks, twice as many warps ended with partly filled queues (193 us).
+// two waves of blocks, twice as many warps ended with partly filled queues (15% later).
 template <int F, int FMT, int PER>
 __global__ void __launch_bounds__(256, kDenseDetBlocks) k_dense_deterministic(Dense3DView g, LookupArgs a) {
   constexpr int T = Filter<F>::T, OFF0 = Filter<F>::OFF0;
@@ -370,9 +372,10 @@ __global__ void __launch_bounds__(256, kDenseDetBlocks) k_dense_deterministic(De
   }
 }
 
-// One thread per query: the trilinear filter (eight scattered voxels: 14.7 M ray-march samples
-// of a 256^3 FP16 grid 100 us in place, 115 us queued; 4 M hits 72 and 84 us), and arrays that
-// are not in this device's memory, whose link bounds the call: a queued kernel writes results
+// One thread per query: the trilinear filter (eight scattered voxels of a 256^3 FP16 grid: 10 M
+// hits 137 us in place, 164 us queued; 8.4 M ray-march samples 48 and 49 us; of 33 M, the most
+// warps' worth, 197 and 182 us, before the live test 236), and arrays that are not in this
+// device's memory, whose link bounds the call: a queued kernel writes results
 // twice and reads coordinates from few warps (4 M hits with results in host memory, trilinear
 // 96 us in place, 514 us queued; tricubic 258 and 590 us).
 template <int F, int FMT>

@@ -14,10 +14,10 @@ int grid_blocks(int64_t n, int threads, int waves = 4);
 // Grid size for kernels whose warps keep queues: at most the blocks that are resident at
 // once (`per_sm` on each SM), so that few warps end with partly filled queues.
 int queue_blocks(int64_t n, int threads, int per_sm);
-// The stochastic dense and sparse kernels launch up to 8 waves of 256-thread blocks.
-// With four queries per thread and the miss shortcut, 8 waves finished the dense
-// benchmark call 3% sooner than 16 and 6% sooner than 32 (2: 11% later; 4 and 6 within
-// 1% of 8, sparse 1-5% slower).  The 2D kernels keep 4 waves (no gain at 16.8M queries,
+// The stochastic dense and sparse kernels without a queue launch up to 8 waves of 256-thread
+// blocks.  With four queries per thread and the miss shortcut, 8 waves finished a ray march
+// (which goes by queue now) 3% sooner than 16 and 6% sooner than 32 (2: 11% later; 4 and 6
+// within 1% of 8, sparse 1-5% slower).  The 2D kernels keep 4 waves (no gain at 16.8M queries,
 // 3% slower at 5.3M with 16).
 constexpr int kStochasticWaves = 8;
 

@@ -49,15 +49,6 @@ __device__ __forceinline__ float2 unpack_h2(uint32_t w) {
 
 // ---------------------------------------------------------------- lookups
 
-// Level of texel storage: returns a pointer to 8 binary16 values of texel (x, y) at
-// level L (latent or fallback; clamp-to-edge).
-__device__ __forceinline__ uint4 neural_texel(const NeuralDev& nd, int L, int x, int y) {
-  const int w = nd.lvl_w[L], h = nd.lvl_h[L];
-  const int cx = min(max(x, 0), w - 1), cy = min(max(y, 0), h - 1);
-  const __half* base = L < nd.nlat ? nd.lat16 : nd.fb16;
-  return __ldg(reinterpret_cast<const uint4*>(base + (nd.lvl_off[L] + (int64_t)cy * w + cx) * 8));
-}
-
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
@@ -132,15 +123,16 @@ __device__ __forceinline__ NeuralPick neural_pick(const NeuralDev& nd, const Loo
 // queries (one per thread) the chosen latent texels are gathered into a shared-memory
 // A tile; one elected thread issues the three layers as tcgen05.mma (M = 128, binary16
 // operands from shared memory, float32 accumulators in tensor memory); after each
-// layer every thread loads its own accumulator row with tcgen05.ld, adds the bias,
-// applies ReLU, rounds to binary16 and writes the next layer's A tile.  Operand tiles
+// layer (its bias included) every thread loads its own accumulator row with tcgen05.ld,
+// applies ReLU, rounds to binary16 and writes the next layer's A operand: layer 2's to a
+// tile in shared memory, layer 3's to tensor memory.  Operand tiles
 // use the no-swizzle K-major layout: 8-row x 16-byte core matrices, core matrices
 // along K 128 bytes apart (LBO), 8-row groups K/8 * 128 bytes apart (SBO).
 
 namespace tc {
 
 constexpr int ROWS = 128;            // queries per tile = threads per group
-constexpr int TMEM_COLS = 128;       // 64 columns per group: D1/D2 in 0..63, D3 in 0..15
+constexpr int TMEM_COLS = 128;       // 64 columns per group: D1/D2 in 0..63, then layer 3's A in 0..31, D3 in 32..47
 constexpr int A1_BYTES = ROWS * 16 * 2, A2_BYTES = ROWS * 64 * 2;
 constexpr int B1_BYTES = 64 * 16 * 2, B2_BYTES = 64 * 64 * 2, B3_BYTES = 16 * 64 * 2;
 
@@ -442,8 +434,8 @@ __device__ __forceinline__ void decode_end(tc::Smem& s, const NeuralDev& nd, int
 }
 
 // Two groups of 128 threads per CTA decode two tiles concurrently: each group owns an
-// A1/A2 tile pair, 64 tensor-memory columns (D1, D2, then D3 over the first 16 once D2
-// has been read), an mbarrier and a named barrier, and walks its own tile sequence;
+// A1/A2 tile pair, 64 tensor-memory columns (D1, D2, then layer 3's A operand and D3), an
+// mbarrier and a named barrier, and walks its own tile sequence;
 // while one group waits on its MMAs or its gathers the other computes.  The weights
 // are shared.  A group's A1 is refilled with the next tile's gather as soon as layer 1
 // has consumed it, and the coordinates of the tile after that are loaded right then, a
@@ -1262,10 +1254,10 @@ __global__ void k_rows_to_h8(const float* src, int cin, __half* dst, int64_t row
 template <class Kernel>
 static cudaError_t launch_decode(Kernel k, OncePerDevice& once, int64_t tiles, const NeuralDev& nd, const LookupArgs& a,
                                  cudaStream_t s) {
-  // at least 46 KiB of shared memory per CTA keeps at most 4 CTAs on an SM (228 KiB),
-  // so their 4 x 128 tensor-memory columns fit in the SM's 512 and no allocation waits
-  const int need = (int)sizeof(tc::Smem) + 1024;
-  const int smem = need > 46 * 1024 ? need : 46 * 1024;
+  // that much shared memory per CTA keeps at most 4 CTAs on an SM (228 KiB), so their
+  // 4 x 128 tensor-memory columns fit in the SM's 512 and no allocation waits
+  constexpr int smem = (int)sizeof(tc::Smem) + 1024;
+  static_assert(smem >= 46 * 1024, "four CTAs on an SM at most");
   const cudaError_t e = once([&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
   if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;

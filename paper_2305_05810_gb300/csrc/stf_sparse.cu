@@ -407,8 +407,8 @@ __global__ void __launch_bounds__(256) k_sparse_stochastic(SparseDev g, LookupAr
 }
 
 // Stochastic lookups of the fixed-window filters, of at most kFastLoopMaxQueries queries,
-// without tap output or permutation.  17 M samples of the 2048^3 cloud, B-spline: 75 us
-// with a chunk's samples in place (17 of 32 lanes active), 58 us by queue, bound by the
+// without tap output or permutation.  17 M samples of the 2048^3 cloud, B-spline: 73 us
+// with a chunk's samples in place (17 of 32 lanes active), 55 us by queue, bound by the
 // latency of the node, leaf and voxel loads.
 constexpr int kSparseQueueBlocks = 6;     // resident 256-thread blocks per SM
 
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(256, kSparseQueueBlocks) k_sparse_stochastic_q
 // lanes were active.  Each warp therefore sorts its samples by what is left to do: those
 // in the box wait in shared memory until 32 can look up their leaves side by side, and
 // those that found a leaf until 32 can sum their taps.  16.8 M samples of the 2048^3 cloud
-// with E4M3 leaves, tricubic: 713 us in place, 168 us queued (79 M instead of 476 M warp
+// with E4M3 leaves, tricubic: 677 us in place, 172 us queued (79 M instead of 476 M warp
 // instructions; each column of four taps one or two aligned 8-byte loads instead of four
 // byte loads).  Four blocks of 64 registers a thread ran 9% sooner than five half-size
 // blocks of 96.

@@ -1,4 +1,5 @@
-"""GPU: the queued deterministic 3D kernels (dense and sparse grids) at the sizes and
+"""GPU: the queued 3D kernels (dense and sparse grids, deterministic and stochastic) and the
+kernels that take their calls without a queue, at the sizes and
 positions where their queues can go wrong: partly filled warps and chunks, misaligned
 arrays, calls on either side of the 128-query chunk limit, windows on the grid's edges,
 across leaves, lower and upper nodes, and next to voxels that are not finite."""
