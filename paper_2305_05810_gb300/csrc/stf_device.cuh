@@ -516,16 +516,20 @@ struct LiveCall {
   bool direct;
 };
 
-// By a block's first warp; a barrier has to follow.
+// The query that a lane of a block's first warp judges by, or NaN where it is not asked for.
 template <int PER>
-__device__ __forceinline__ void stage_live(const LookupArgs& a, const LiveBox& box, LiveCall& s) {
+__device__ __forceinline__ void load_sample(const LookupArgs& a, float (&x)[3]) {
+  x[0] = x[1] = x[2] = __int_as_float(0x7fc00000);
+  if (PER != 4 || threadIdx.x >= 32 || !quad_loop3_ok(a)) return;
+  const float* p = a.coords + 3 * __umulhi(threadIdx.x * 2654435769u, (uint32_t)a.n);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) x[d] = __ldg(p + d);
+}
+
+// From those; a barrier has to follow.
+__device__ __forceinline__ void stage_live(const LiveBox& box, const float (&x)[3], LiveCall& s) {
   if (threadIdx.x >= 32) return;
-  bool direct = false;
-  if (PER == 4 && quad_loop3_ok(a)) {
-    const float* p = a.coords + 3 * __umulhi(threadIdx.x * 2654435769u, (uint32_t)a.n);
-    const float x[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
-    direct = __popc(__ballot_sync(0xffffffffu, box.has(x))) >= 24;
-  }
+  const bool direct = __popc(__ballot_sync(0xffffffffu, box.has(x))) >= 24;
   if (threadIdx.x == 0) s = {box, direct};
 }
 

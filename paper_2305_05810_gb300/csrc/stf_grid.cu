@@ -98,7 +98,9 @@ __global__ void __launch_bounds__(256, kDenseQueueBlocks) k_dense_stochastic_que
   __shared__ LiveQueue<PER> queues[8];
   __shared__ LiveCall call;
   const int zero[3] = {0, 0, 0}, dims[3] = {g.nx, g.ny, g.nz};
-  stage_live<PER>(a, live_box(zero, dims, W::LO, W::HI), call);
+  float sample[3];
+  load_sample<PER>(a, sample);
+  stage_live(live_box(zero, dims, W::LO, W::HI), sample, call);
   __syncthreads();
   if (PER == 4 && call.direct) {
     const MissBox mb = miss_box<F>(0, 0, 0, g.nx, g.ny, g.nz);

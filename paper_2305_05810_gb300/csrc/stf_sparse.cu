@@ -309,7 +309,7 @@ __device__ __forceinline__ float sparse_value(const SparseDev& g, int64_t leaf, 
   }
 }
 
-__device__ __forceinline__ void stage_upper(const SparseDev& g, UpperSmem& su) {
+__device__ __forceinline__ void stage_upper_nodes(const SparseDev& g, UpperSmem& su) {
   if (g.n_upper > 0) {
     for (int k = threadIdx.x; k < 512; k += blockDim.x) {
       su.mask[k] = __ldg(g.upper_mask + k);
@@ -317,6 +317,10 @@ __device__ __forceinline__ void stage_upper(const SparseDev& g, UpperSmem& su) {
     }
   }
   if (threadIdx.x < 3) su.origin[threadIdx.x] = g.n_upper > 0 ? __ldg(g.upper_origin + threadIdx.x) : INT_MIN;
+}
+
+__device__ __forceinline__ void stage_upper(const SparseDev& g, UpperSmem& su) {
+  stage_upper_nodes(g, su);
   __syncthreads();
 }
 
@@ -418,8 +422,11 @@ __global__ void __launch_bounds__(256, kSparseQueueBlocks) k_sparse_stochastic_q
   __shared__ UpperSmem su;
   __shared__ LiveQueue<PER> queues[8];
   __shared__ LiveCall call;
-  stage_live<PER>(a, live_box(g.bb_lo, g.bb_hi, W::LO, W::HI), call);
-  stage_upper(g, su);                                // (ends with a barrier)
+  float sample[3];
+  load_sample<PER>(a, sample);                       // (under way while the nodes are staged)
+  stage_upper_nodes(g, su);
+  stage_live(live_box(g.bb_lo, g.bb_hi, W::LO, W::HI), sample, call);
+  __syncthreads();
   if (PER == 4 && call.direct) {
     const MissBox mb = miss_box<F>(g.bb_lo[0], g.bb_lo[1], g.bb_lo[2], g.bb_hi[0], g.bb_hi[1], g.bb_hi[2]);
     // (whole rounds of four; a last round for some threads only would hold up the rest)
